@@ -381,6 +381,10 @@ iesh_status iesh_create(iesh_ctx **out, const iesh_model *model, const iesh_opti
     A(d.cheb, T * kChebStride)
     if (opt->propagator == IESH_PROP_AVERAGED && !opt->no_deflation)
         A(d.defl, T * (size_t)defl_stride(N, Ne))
+    if (!ctx->mixed && opt->propagator == IESH_PROP_AVERAGED && cheb_fx_eligible(N, Ne)) {
+        d.fx_work_bytes = cheb_fx_work_bytes(N, Ne, max_traj);
+        A(d.fx_work, d.fx_work_bytes)
+    }
     A(ctx->live, T)
     A(ctx->n_live, 1)
     A(ctx->obs, 4 * T)
@@ -408,6 +412,7 @@ iesh_status iesh_create(iesh_ctx **out, const iesh_model *model, const iesh_opti
     configure_hop_smem();
     configure_cheb_tc();
     configure_cheb_tc16();
+    configure_cheb_fx();
     {
         std::vector<float> ed((size_t)M * M);
         for (int a = 0; a < M; ++a)

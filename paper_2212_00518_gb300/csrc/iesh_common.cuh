@@ -81,6 +81,9 @@ struct DevState {
     // kernel shapes (0 = built-in choice): propagator electrons per thread
     // and column groups per CTA, threads of the hop kernel
     int cheb_ept, cheb_G, hop_threads;
+    // workspace of the FP64 tensor-core propagator (one slot per CTA), or null
+    unsigned char *fx_work;
+    size_t fx_work_bytes;
     // two adsorbate orbitals over six nuclear coordinates: x, p, F and vprev
     // are [n][6]; q0 holds the components Q_0j on orbital 0 and q2 the
     // components Q_1j on orbital 1; geo2 [n][8] holds h_0, h_1 and, with the

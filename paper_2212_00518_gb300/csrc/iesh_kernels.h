@@ -66,6 +66,12 @@ size_t cheb_tc16_smem_bytes(int N, int Ne);
 bool cheb_tc16_eligible(int N, int Ne);
 void configure_cheb_tc16();
 cudaError_t launch_cheb_tc16(const DevState &s, double dt, cudaStream_t st);
+// FP64 propagator on the tensor cores (digits of fixed-point numbers as FP16,
+// N <= 256); its workspace is made with the context
+bool cheb_fx_eligible(int N, int Ne);
+size_t cheb_fx_work_bytes(int N, int Ne, int64_t max_traj);
+void configure_cheb_fx();
+cudaError_t launch_cheb_fx(const DevState &s, double dt, cudaStream_t st);
 // unitarity check of the coefficient columns (sets ST_NORM), observables
 // out[4][n] = (kinetic energy, potential energy, occupied-surface and
 // wavefunction impurity populations), batch status summary out[9]

@@ -233,11 +233,15 @@ constexpr double kDeflAmp64 = 1e3, kDeflAmp32 = 16.0;
 // Thread 0 has set up the series over the bulk interval; it keeps the
 // deflation if the series amplifies the u direction by at most amp, else it
 // sets the full interval up.  Returns the block-uniform decision.
+// rtop: the top row's Gershgorin radius.  The FP64 propagator's fixed-point
+// ranges also ask that the top row's couplings and diagonal stay within 8 and
+// 10^6 bulk half-widths (rows inside the interval have at most 1).
 __device__ inline bool defl_keep(const DevState &s, int64_t t, bool deflate, double mu, double lo, double hi,
-                                 double tol, double amp, double *df, int *flag)
+                                 double tol, double amp, double rtop, double *df, int *flag)
 {
     if (threadIdx.x == 0) {
-        bool k = deflate && cheb_amplification(s.cheb + t * kChebStride, mu) <= amp;
+        const double *cb = s.cheb + t * kChebStride;
+        bool k = deflate && cheb_amplification(cb, mu) <= amp && rtop <= 8.0 * cb[1] && mu - cb[0] <= 1e6 * cb[1];
         if (deflate && !k) cheb_setup(s, t, lo, hi, tol);
         *flag = k;
         if (df) {
@@ -361,7 +365,7 @@ __global__ void __launch_bounds__(256) k_build_w(DevState s, double dt, double m
     }
     if (threadIdx.x == 0) cheb_setup(s, t, lo, hb, tol);
     __shared__ int keep;
-    if (!defl_keep(s, t, deflate, mu, lo, hi, tol, kDeflAmp64, df, &keep)) return;
+    if (!defl_keep(s, t, deflate, mu, lo, hi, tol, kDeflAmp64, deflate ? Lk_s[N - 1] - hb_s[N - 1] : 0.0, df, &keep)) return;
     const int Ne = s.Ne;
     double *q = df + kDeflHead;
     for (int j = threadIdx.x; j < N; j += blockDim.x) {
@@ -550,7 +554,7 @@ __global__ void __launch_bounds__(256, 5) k_build_w_f32(DevState s, double dt, d
     if (threadIdx.x == 0) cheb_setup(s, t, lo, hb, tol);
     if (!dfl) return;
     __shared__ int keep;
-    if (!defl_keep(s, t, deflate, mu, lo, hi, tol, kDeflAmp32, df, &keep)) return;
+    if (!defl_keep(s, t, deflate, mu, lo, hi, tol, kDeflAmp32, 0.0, df, &keep)) return;
     const int Ne = s.Ne;
     float *q = reinterpret_cast<float *>(df + kDeflHead);  // packed floats
     for (int j = threadIdx.x; j < N; j += blockDim.x) {
@@ -1645,6 +1649,8 @@ cudaError_t launch_cheb(const DevState &s, double dt, bool mixed, cudaStream_t s
         }
         return cudaSuccess;
     }
+    // tensor cores where cheb_fx_eligible (the context then has the workspace)
+    if (s.fx_work) return launch_cheb_fx(s, dt, st);
     int ept, G;
     cheb_shape(s.N, s.Ne, ept, G);
     if (s.cheb_ept > 0 && s.cheb_G > 0) {

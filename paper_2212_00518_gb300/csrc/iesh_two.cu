@@ -1304,6 +1304,10 @@ iesh_status iesh2_create(iesh2_ctx **out, const iesh2_model *model, int precisio
     A2(d.status, T) A2(d.nstep, T) A2(d.hops, T) A2(d.frus, T)
     A2(d.scratch, T * (size_t)d.scratch_stride)
     A2(d.cheb, T * kChebStride)
+    if (!ctx->mixed && cheb_fx_eligible(N, Ne)) {
+        d.fx_work_bytes = cheb_fx_work_bytes(N, Ne, max_traj);
+        A2(d.fx_work, d.fx_work_bytes)
+    }
     double *mu_d = nullptr;
     float2 *ppdf_d = nullptr;
     if (ctx->nested) A2(mu_d, T * (size_t)(M + 1))
@@ -1320,6 +1324,7 @@ iesh_status iesh2_create(iesh2_ctx **out, const iesh2_model *model, int precisio
     configure_hop_smem();
     configure_cheb_tc();
     configure_cheb_tc16();
+    configure_cheb_fx();
     // the slots of the eigen kernel can pass the 48 KiB default (N near 65)
     CU2(cudaFuncSetAttribute(k2_eigen<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)eigen2_smem(N, M, eigen_tpb(N), false)));
