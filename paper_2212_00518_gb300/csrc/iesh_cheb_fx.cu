@@ -182,12 +182,6 @@ __device__ __forceinline__ float abs_float(double x)
     return __int_as_float(((h - (896 << 20)) << 3) | (int)((uint32_t)__double2loint(x) >> 29));
 }
 
-__device__ __forceinline__ bool elect_one()
-{
-    uint32_t p;
-    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(p));
-    return p != 0;
-}
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint64_t *mbar)
 {
     const uint32_t mb = tc::smem_addr(mbar);
@@ -586,7 +580,7 @@ __global__ void __launch_bounds__(kFxThreads, 1)
                 __syncthreads();  // T's digits are in place, D has been read
                 tc::fence_after_sync();
                 if (warp == 0) {
-                    if (elect_one()) {
+                    if (tc::elect_one()) {
                         switch (nsl) {
                         case 4: ok = fx_order<4>(m, fpar, !resident || ord == 0, !resident); break;
                         case 5: ok = fx_order<5>(m, fpar, !resident || ord == 0, !resident); break;
@@ -597,7 +591,7 @@ __global__ void __launch_bounds__(kFxThreads, 1)
                     }
                     __syncwarp();
                 } else if (warp == 5) {
-                    if (elect_one()) {
+                    if (tc::elect_one()) {
                         // this order's stages and the next order's first ones, as slots free up
                         const uint32_t upto = (uint32_t)((ord + 1) * nstage + nst - 1);
                         for (; qp < qend && qp < upto; ++qp) {

@@ -38,6 +38,8 @@ struct iesh_eocc_ctx {
     int M = 0, Ne = 0;
     double *eps_d = nullptr, *w_d = nullptr;  // bath energies, weights (FP64)
     float *eps_f = nullptr, *w_f = nullptr;   // FP32 copies
+    float2 *eps_df = nullptr;                 // energies as double-float pairs
+    double wsum = 0.0;                        // sum of the weights
     std::string err;
 };
 
@@ -75,81 +77,132 @@ __device__ __forceinline__ Ads<R> ads_eval(const EoccConst &k, const R *x, const
     return o;
 }
 
-// One CTA per geometry, one thread per needed root (the Ne lowest).
+// The geometry's two-level block: one thread forms it (an FP64 instruction
+// costs a warp 64 cycles of its scheduler's FP64 pipe whatever its active
+// lanes, and the exponentials are dozens of them).
+template <class R>
+struct EoccGeo {
+    Ads<R> ad;
+    R c2, rc, hp, hm, tt;  // |c|^2, 1/|c|, h_+, h_-, t
+    int pos;               // bath energies below h_-
+};
+
+// One CTA per geometry, one thread per needed root (the Ne lowest).  FP64:
+// the roots are found in stages, FP32 and double-float sums before one FP64
+// evaluation (secular_root); the poles and weights are kept in double-float
+// beside the FP64 ones.
 template <class R>
 __global__ void k_eocc_fwd(int64_t B, int M, int Ne, EoccConst kc, const R *__restrict__ eps,
-                           const R *__restrict__ w, const R *__restrict__ x, const R *__restrict__ th,
-                           R *__restrict__ E, R *__restrict__ saved, uint32_t *__restrict__ status)
+                           const R *__restrict__ w, const float2 *__restrict__ epsdf, R wsum, const R *__restrict__ x,
+                           const R *__restrict__ th, R *__restrict__ E, R *__restrict__ saved,
+                           uint32_t *__restrict__ status)
 {
+    constexpr bool kF64 = sizeof(R) == 8;
     extern __shared__ __align__(16) unsigned char eocc_smem[];
-    R *pole = reinterpret_cast<R *>(eocc_smem);  // [M + 1]
-    R *wt = pole + (M + 1);                      // [M + 1]
-    double *red = reinterpret_cast<double *>(wt + (M + 1));  // [32], 2(M+1) values before it
+    double *red = reinterpret_cast<double *>(eocc_smem);      // [5][blockDim.x]
+    R *pole = reinterpret_cast<R *>(red + 5 * blockDim.x);    // [M + 1]
+    R *wt = pole + (M + 1);                                   // [M + 1]
+    float2 *pdf = reinterpret_cast<float2 *>(wt + (M + 1));   // [M + 1] (FP64)
+    float2 *wdf = pdf + (M + 1);                              // [M + 1] (FP64)
+    __shared__ EoccGeo<R> gs;
     const int64_t b = blockIdx.x;
     if (b >= B) return;
-    R xs[6], ths[16];
-    for (int q = 0; q < 6; ++q) xs[q] = x[b * 6 + q];
-    for (int q = 0; q < 16; ++q) ths[q] = th[q];
-    const Ads<R> ad = ads_eval<R>(kc, xs, ths);
-    const R c2 = ad.c[0] * ad.c[0] + ad.c[1] * ad.c[1];
-    const R c = sqrt(c2);
-    const R hp = (ad.c[0] * ad.c[0] * ad.h[0] + ad.c[1] * ad.c[1] * ad.h[1]) / c2;
-    const R hm = (ad.c[1] * ad.c[1] * ad.h[0] + ad.c[0] * ad.c[0] * ad.h[1]) / c2;
-    const R tt = ad.c[0] * ad.c[1] * (ad.h[1] - ad.h[0]) / c2;
+    if (threadIdx.x == 0) {
+        R xs[6], ths[16];
+        for (int q = 0; q < 6; ++q) xs[q] = x[b * 6 + q];
+        for (int q = 0; q < 16; ++q) ths[q] = th[q];
+        const Ads<R> ad = ads_eval<R>(kc, xs, ths);
+        const R c2 = ad.c[0] * ad.c[0] + ad.c[1] * ad.c[1];
+        const R hm = (ad.c[1] * ad.c[1] * ad.h[0] + ad.c[0] * ad.c[0] * ad.h[1]) / c2;
+        gs.ad = ad;
+        gs.c2 = c2;
+        gs.rc = R(1) / sqrt(c2);
+        gs.hp = (ad.c[0] * ad.c[0] * ad.h[0] + ad.c[1] * ad.c[1] * ad.h[1]) / c2;
+        gs.hm = hm;
+        gs.tt = ad.c[0] * ad.c[1] * (ad.h[1] - ad.h[0]) / c2;
+        int lo = 0, hi = M;  // ascending energies: bisection
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (eps[mid] < hm) lo = mid + 1;
+            else hi = mid;
+        }
+        gs.pos = lo;
+    }
+    __syncthreads();
+    const R c2 = gs.c2, hp = gs.hp, hm = gs.hm, tt = gs.tt;
     const bool decoupled = !(tt * tt > R(0));
     // poles: bath energies, plus h_- in its sorted place unless |-> decouples
-    int pos = 0;
-    for (int k = 0; k < M; ++k) pos += (eps[k] < hm);
+    const int pos = gs.pos;
     const int P = decoupled ? M : M + 1;
     for (int k = threadIdx.x; k < M; k += blockDim.x) {
         const int slot = (decoupled || k < pos) ? k : k + 1;
+        const R wk = c2 * w[k];
         pole[slot] = eps[k];
-        wt[slot] = c2 * w[k];
+        wt[slot] = wk;
+        if constexpr (kF64) {
+            const dfl d = dfl_from(wk);
+            pdf[slot] = epsdf[k];
+            wdf[slot] = make_float2(d.hi, d.lo);
+        }
     }
     if (!decoupled && threadIdx.x == 0) {
         pole[pos] = hm;
         wt[pos] = tt * tt;
-    }
-    __syncthreads();
-    R Z2 = 0;
-    for (int k = 0; k < P; ++k) Z2 += wt[k];
-    uint32_t st = 0;
-    double le = 0.0, s0 = 0.0, s1 = 0.0, t0 = 0.0, t1 = 0.0;
-    const int r = threadIdx.x;
-    if (r < Ne) {
-        R lam, qp;
-        const Poles<R> pp = {P, pole, wt, nullptr, nullptr, nullptr};
-        secular_root<R>(r, pp, hp, Z2, false, R(0), lam, qp, st);
-        const R qm = decoupled ? R(0) : tt * qp / (lam - hm);
-        const R Q0 = (ad.c[0] * qp - ad.c[1] * qm) / c;
-        const R Q1 = (ad.c[1] * qp + ad.c[0] * qm) / c;
-        le = (double)lam;
-        s0 = (double)(Q0 * Q0);
-        s1 = (double)(Q1 * Q1);
-        t0 = (double)(Q0 * Q0 * (lam - ad.h[0]));
-        t1 = (double)(Q1 * Q1 * (lam - ad.h[1]));
-        if (decoupled && r == Ne - 1 && hm < lam) {
-            // the decoupled |-> state is among the Ne lowest: it replaces root Ne-1
-            le = (double)hm;
-            const R P0 = -ad.c[1] / c, P1 = ad.c[0] / c;
-            s0 = (double)(P0 * P0);
-            s1 = (double)(P1 * P1);
-            t0 = (double)(P0 * P0 * (hm - ad.h[0]));
-            t1 = (double)(P1 * P1 * (hm - ad.h[1]));
+        if constexpr (kF64) {
+            const dfl d = dfl_from(hm), d2 = dfl_from(tt * tt);
+            pdf[pos] = make_float2(d.hi, d.lo);
+            wdf[pos] = make_float2(d2.hi, d2.lo);
         }
     }
+    __syncthreads();
+    const R Z2 = c2 * wsum + (decoupled ? R(0) : tt * tt);
+    uint32_t st = 0;
+    R v[5] = {0, 0, 0, 0, 0};  // lam, Q_0^2, Q_1^2, Q_a^2 (lam - h_a)
+    const int r = threadIdx.x;
+    if (r < Ne) {
+        R lam, qp, tau;
+        int o;
+        if constexpr (kF64) {
+            const Poles<R> pp = {P, pole, wt, nullptr, nullptr, wdf, 0, -1, R(0), pdf, nullptr};
+            secular_root<R, EV_PLAIN, EV_POLE_DF, EV_POLE_F32>(r, pp, hp, Z2, false, R(0), lam, qp, st, &o, &tau);
+        } else {
+            const Poles<R> pp = {P, pole, wt, nullptr, nullptr, nullptr};
+            secular_root<R>(r, pp, hp, Z2, false, R(0), lam, qp, st, &o, &tau);
+        }
+        // lam - h_-: the exact offset when the origin pole is h_- itself
+        const R qm = decoupled ? R(0) : tt * qp / (o == pos ? tau : (pole[o] - hm) + tau);
+        const Ads<R> &ad = gs.ad;
+        R Q0 = (ad.c[0] * qp - ad.c[1] * qm) * gs.rc;
+        R Q1 = (ad.c[1] * qp + ad.c[0] * qm) * gs.rc;
+        if (decoupled && r == Ne - 1 && hm < lam) {
+            // the decoupled |-> state is among the Ne lowest: it replaces root Ne-1
+            lam = hm;
+            Q0 = -ad.c[1] * gs.rc;
+            Q1 = ad.c[0] * gs.rc;
+        }
+        v[0] = lam;
+        v[1] = Q0 * Q0;
+        v[2] = Q1 * Q1;
+        v[3] = v[1] * (lam - ad.h[0]);
+        v[4] = v[2] * (lam - ad.h[1]);
+    }
     if (st) atomicOr(&status[b], st);
-    le = block_sum(le, red);
-    s0 = block_sum(s0, red);
-    s1 = block_sum(s1, red);
-    t0 = block_sum(t0, red);
-    t1 = block_sum(t1, red);
-    if (threadIdx.x == 0) {
-        E[b] = (R)le;
-        saved[b * 4 + 0] = (R)s0;
-        saved[b * 4 + 1] = (R)s1;
-        saved[b * 4 + 2] = (R)t0;
-        saved[b * 4 + 3] = (R)t1;
+    // the five sums in FP64: warp w takes sum w, fixed order (each thread
+    // adding its five into butterflies of its own would be 25 FP64
+    // instructions per warp instead of at most 10)
+#pragma unroll
+    for (int q = 0; q < 5; ++q) red[q * blockDim.x + threadIdx.x] = (double)v[q];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int q = warp; q < 5; q += nw) {
+        double a = red[q * blockDim.x + lane];
+        for (int i = lane + 32; i < (int)blockDim.x; i += 32) a += red[q * blockDim.x + i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (lane == 0) {
+            if (q == 0) E[b] = (R)a;
+            else saved[b * 4 + q - 1] = (R)a;
+        }
     }
 }
 
@@ -289,15 +342,22 @@ iesh_status iesh_eocc_create(iesh_eocc_ctx **out, const iesh_eocc_model *model, 
         w.push_back(0.5 * (model->band_hi - model->mu) * wl[k]);
     }
     std::vector<float> epsf(eps.begin(), eps.end()), wf(w.begin(), w.end());
+    std::vector<float2> epsdf(M);
+    for (int k = 0; k < M; ++k) {
+        epsdf[k] = make_float2(epsf[k], (float)(eps[k] - (double)epsf[k]));
+        c->wsum += w[k];
+    }
     if (cudaMalloc(&c->eps_d, M * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&c->w_d, M * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&c->eps_f, M * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&c->w_f, M * sizeof(float)) != cudaSuccess)
+        cudaMalloc(&c->w_f, M * sizeof(float)) != cudaSuccess ||
+        cudaMalloc(&c->eps_df, M * sizeof(float2)) != cudaSuccess)
         return efail(c, IESH_ENOMEM, "cudaMalloc failed");
     if (cudaMemcpy(c->eps_d, eps.data(), M * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(c->w_d, w.data(), M * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(c->eps_f, epsf.data(), M * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(c->w_f, wf.data(), M * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)
+        cudaMemcpy(c->w_f, wf.data(), M * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(c->eps_df, epsdf.data(), M * sizeof(float2), cudaMemcpyHostToDevice) != cudaSuccess)
         return efail(c, IESH_ECUDA, "bath upload failed");
     return IESH_OK;
 }
@@ -309,6 +369,7 @@ iesh_status iesh_eocc_destroy(iesh_eocc_ctx *c)
     cudaFree(c->w_d);
     cudaFree(c->eps_f);
     cudaFree(c->w_f);
+    cudaFree(c->eps_df);
     delete c;
     return IESH_OK;
 }
@@ -328,14 +389,28 @@ iesh_status iesh_eocc_forward(iesh_eocc_ctx *c, int64_t B, int precision, const 
     cudaError_t e = cudaMemsetAsync(status, 0, B * sizeof(uint32_t), c->stream);
     if (e != cudaSuccess) return efail(c, IESH_ECUDA, cudaGetErrorString(e));
     if (precision == IESH_PREC_FP64) {
-        const size_t smem = (size_t)2 * (M + 2) * sizeof(double) + 32 * sizeof(double);
+        const size_t smem = (size_t)5 * threads * sizeof(double) + (size_t)(M + 1) * (2 * sizeof(double) + 2 * sizeof(float2));
+        if (smem > 48 * 1024) {  // a process-wide function attribute: only raised
+            cudaFuncAttributes fa;
+            e = cudaFuncGetAttributes(&fa, k_eocc_fwd<double>);
+            if (e == cudaSuccess && fa.maxDynamicSharedSizeBytes < (int)smem)
+                e = cudaFuncSetAttribute(k_eocc_fwd<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return efail(c, IESH_ECUDA, cudaGetErrorString(e));
+        }
         k_eocc_fwd<double><<<(unsigned)B, threads, smem, c->stream>>>(
-            B, M, Ne, kc, c->eps_d, c->w_d, (const double *)x, (const double *)theta, (double *)E,
+            B, M, Ne, kc, c->eps_d, c->w_d, c->eps_df, c->wsum, (const double *)x, (const double *)theta, (double *)E,
             (double *)saved, status);
     } else if (precision == IESH_PREC_MIXED) {
-        const size_t smem = (size_t)2 * (M + 2) * sizeof(float) + 33 * sizeof(double);
+        const size_t smem = (size_t)5 * threads * sizeof(double) + (size_t)2 * (M + 1) * sizeof(float);
+        if (smem > 48 * 1024) {
+            cudaFuncAttributes fa;
+            e = cudaFuncGetAttributes(&fa, k_eocc_fwd<float>);
+            if (e == cudaSuccess && fa.maxDynamicSharedSizeBytes < (int)smem)
+                e = cudaFuncSetAttribute(k_eocc_fwd<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return efail(c, IESH_ECUDA, cudaGetErrorString(e));
+        }
         k_eocc_fwd<float><<<(unsigned)B, threads, smem, c->stream>>>(
-            B, M, Ne, kc, c->eps_f, c->w_f, (const float *)x, (const float *)theta, (float *)E,
+            B, M, Ne, kc, c->eps_f, c->w_f, c->eps_df, (float)c->wsum, (const float *)x, (const float *)theta, (float *)E,
             (float *)saved, status);
     } else {
         return efail(c, IESH_EINVAL, "unknown precision");

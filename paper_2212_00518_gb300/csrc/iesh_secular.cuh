@@ -48,6 +48,16 @@ __device__ __forceinline__ double pole_recip<double>(double d)
     return fma(r, fma(e, e, e), r);
 }
 
+// FP32: the approximate reciprocal (1 ulp) and one Newton step, in place of a
+// correctly rounded division's eight or so instructions.
+template <>
+__device__ __forceinline__ float pole_recip<float>(float d)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return fmaf(r, fmaf(-d, r, 1.0f), r);
+}
+
 // Double-float numbers (hi + lo, two FP32 values, about 48 significant bits)
 // for the secular sums of the mixed-precision path: the FP32 pipe is 64x
 // wider than the FP64 pipe on this part.  Error-free transformations:
@@ -80,13 +90,23 @@ __device__ __forceinline__ dfl dfl_mul(dfl a, dfl b)
     e = fmaf(a.lo, b.hi, e);
     return dfl_fast_two_sum(p, e);
 }
-// 1/a: the rounded FP32 reciprocal r0 corrected by r0 (1 - a r0)
+// 1/a: the FP32 reciprocal estimate r0 (1 ulp) corrected by r0 (e + e^2), e =
+// 1 - a r0
 __device__ __forceinline__ dfl dfl_rcp(dfl a)
 {
-    const float r0 = __frcp_rn(a.hi);
+    float r0;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(a.hi));
     float e = fmaf(-a.hi, r0, 1.0f);
     e = fmaf(-a.lo, r0, e);
-    return dfl_fast_two_sum(r0, r0 * e);
+    return dfl_fast_two_sum(r0, r0 * fmaf(e, e, e));
+}
+// a += b with the low parts summed on their own (renormalised once, by
+// dfl_value or dfl_add, at the end of a sum)
+__device__ __forceinline__ void dfl_acc(dfl &a, dfl b)
+{
+    const dfl s = dfl_two_sum(a.hi, b.hi);
+    a.hi = s.hi;
+    a.lo += s.lo + b.lo;
 }
 __device__ __forceinline__ dfl dfl_from(double x)
 {
@@ -107,6 +127,8 @@ __device__ __forceinline__ double dfl_value(dfl a) { return (double)a.hi + (doub
 // [nb][nb], hdf[k] = tau_k as a double-float pair and ob[k] its bath pole,
 // so mu_o - mu_k = (eps_{ob[o]} - eps_{ob[k]}) + (tau_o - tau_k) keeps its
 // relative accuracy however close the two roots are.
+// EV_POLE_DF and EV_POLE_F32 (starting stages): the poles themselves as
+// double-float pairs in hdf; the differences are formed per term.
 template <class R>
 struct Poles {
     int M;
@@ -120,9 +142,10 @@ struct Poles {
 
 // Evaluation modes of the secular sums: EV_PLAIN (eps_o - eps_k formed per
 // term), EV_TABLE (FP64 table), EV_DFLOAT (double-float sums on the FP32
-// pipe; the origin term and everything outside the sums stay FP64), EV_TWO_DF
-// and EV_NESTED (double-float, see Poles).
-enum { EV_PLAIN = 0, EV_TABLE = 1, EV_DFLOAT = 2, EV_TWO_DF = 3, EV_NESTED = 4 };
+// pipe; the origin term and the assembly of g stay FP64), EV_TWO_DF,
+// EV_NESTED and EV_POLE_DF (double-float, see Poles), EV_POLE_F32 (FP32 sums).
+enum { EV_PLAIN = 0, EV_TABLE = 1, EV_DFLOAT = 2, EV_TWO_DF = 3, EV_NESTED = 4, EV_POLE_DF = 5, EV_POLE_F32 = 6 };
+__host__ __device__ constexpr bool ev_is_df(int ev) { return ev == EV_DFLOAT || ev == EV_TWO_DF || ev == EV_NESTED || ev == EV_POLE_DF; }
 
 // mu_o - mu_k + td for the nested poles (EV_NESTED), in double-float.
 template <class R>
@@ -143,102 +166,95 @@ __device__ __forceinline__ dfl nested_gap(const Poles<R> &P, int o, int k, dfl t
 // z_k q0 / (lam - eps_k).  Each root is found in the shifted variable
 // tau = lam - eps_o relative to its nearer pole o, so lam - eps_k =
 // (eps_o - eps_k) + tau keeps full relative accuracy.
+// gp = gp_rest + the origin's share; s3 = sum_k z_k^2 / (lam - eps_k)^3
+// (FP32, where the mode forms it), so g'' = -2 s3; sabs = the scale of g's
+// rounding error.
 template <class R>
 struct Sec {
     R g, gp, gp_rest, qo, sabs;
+    float s3;
 };
 
-// With ABS the sum of |z_k^2 / (lam - eps_k)| over k != o (the scale of the
-// rounding error of g, for the stopping test) is accumulated into e.sabs;
-// without it e.sabs is left at zero for the caller to fill in.  EV selects
-// how the sums over k != o are formed (see EV_*); the terms k != o have
-// |lam - eps_k| >= half a pole gap, so their double-float range is safe.
+// With ABS the sum of |z_k^2 / (lam - eps_k)| over k != o is accumulated into
+// e.sabs; without it e.sabs is left at zero for the caller to fill in (the
+// FP32 and double-float modes form it in FP32 along the way).  EV selects how
+// the sums over k != o are formed (see EV_*); the terms k != o have |lam -
+// eps_k| >= half a pole gap, so their double-float range is safe.
 template <class R, bool ABS, int EV>
 __device__ __forceinline__ Sec<R> sec_eval(const Poles<R> &P, int o, R tau, R eomh)
 {
     const int M = P.M;
     R s1 = 0, s2 = 0, sa = 0;
-    if constexpr (EV == EV_DFLOAT) {
+    float s3 = 0.f;
+    if constexpr (ev_is_df(EV)) {
         // two accumulator sets (even and odd poles), added at the end: the
         // double-float additions are a serial chain, two chains run at once
         const dfl td = dfl_from((double)tau);
-        dfl d1[2] = {{0.f, 0.f}, {0.f, 0.f}}, d2[2] = {{0.f, 0.f}, {0.f, 0.f}}, da[2] = {{0.f, 0.f}, {0.f, 0.f}};
+        dfl d1[2] = {{0.f, 0.f}, {0.f, 0.f}}, d2[2] = {{0.f, 0.f}, {0.f, 0.f}};
+        float da = 0.f;
+        const bool oh = EV == EV_TWO_DF && o == P.hpos;
+        const int ob = EV != EV_TWO_DF ? 0 : (oh ? 0 : ((P.hpos >= 0 && o > P.hpos) ? o - 1 : o));
+        const float2 po = EV == EV_POLE_DF ? P.hdf[o] : make_float2(0.f, 0.f);
         auto term = [&](int k, int h) {
-            const float2 dk = P.ddf[(size_t)k * M + o], zk = P.z2df[k];
-            const dfl r = dfl_rcp(dfl_add({dk.x, dk.y}, td));  // 1 / (lam - eps_k)
-            const dfl q = dfl_mul({zk.x, zk.y}, r);
-            if (k != o) {
-                d1[h] = dfl_add(d1[h], q);
-                d2[h] = dfl_add(d2[h], dfl_mul(q, r));
-                if (ABS) da[h] = dfl_add(da[h], q.hi < 0.f ? dfl{-q.hi, -q.lo} : q);
+            int q = k;  // index of the weight
+            dfl x;      // lam - eps_k
+            if constexpr (EV == EV_DFLOAT) {
+                const float2 dk = P.ddf[(size_t)k * M + o];
+                x = dfl_add({dk.x, dk.y}, td);
+            } else if constexpr (EV == EV_TWO_DF) {
+                q = (P.hpos >= 0 && k >= P.hpos) ? k + 1 : k;
+                const float2 dk = oh ? P.hdf[k] : P.ddf[(size_t)k * P.nb + ob];
+                x = dfl_add({dk.x, dk.y}, td);
+            } else if constexpr (EV == EV_NESTED) {
+                if (k == o) return;
+                x = nested_gap(P, o, k, td);
+            } else {
+                const float2 pk = P.hdf[k];
+                x = dfl_add(dfl_add({po.x, po.y}, {-pk.x, -pk.y}), td);
             }
-        };
-        int k = 0;
-        for (; k + 1 < M; k += 2) {
-            term(k, 0);
-            term(k + 1, 1);
-        }
-        if (k < M) term(k, 0);
-        s1 = (R)dfl_value(dfl_add(d1[0], d1[1]));
-        s2 = (R)dfl_value(dfl_add(d2[0], d2[1]));
-        sa = (R)dfl_value(dfl_add(da[0], da[1]));
-    } else if constexpr (EV == EV_NESTED) {
-        // two accumulator sets, as above
-        const dfl td = dfl_from((double)tau);
-        dfl d1[2] = {{0.f, 0.f}, {0.f, 0.f}}, d2[2] = {{0.f, 0.f}, {0.f, 0.f}}, da[2] = {{0.f, 0.f}, {0.f, 0.f}};
-        auto term = [&](int k, int h) {
-            if (k == o) return;
-            const dfl r = dfl_rcp(nested_gap(P, o, k, td));  // 1 / (lam - mu_k)
-            const float2 zk = P.z2df[k];
-            const dfl q = dfl_mul({zk.x, zk.y}, r);
-            d1[h] = dfl_add(d1[h], q);
-            d2[h] = dfl_add(d2[h], dfl_mul(q, r));
-            if (ABS) da[h] = dfl_add(da[h], q.hi < 0.f ? dfl{-q.hi, -q.lo} : q);
-        };
-        int k = 0;
-        for (; k + 1 < M; k += 2) {
-            term(k, 0);
-            term(k + 1, 1);
-        }
-        if (k < M) term(k, 0);
-        s1 = (R)dfl_value(dfl_add(d1[0], d1[1]));
-        s2 = (R)dfl_value(dfl_add(d2[0], d2[1]));
-        sa = (R)dfl_value(dfl_add(da[0], da[1]));
-    } else if constexpr (EV == EV_TWO_DF) {
-        // bath poles in double-float from the bath table (origin a bath pole)
-        // or from hdf (origin h_-); the h_- term itself in R.  Two
-        // accumulator sets, as above
-        const dfl td = dfl_from((double)tau);
-        const bool oh = o == P.hpos;
-        const int ob = oh ? 0 : ((P.hpos >= 0 && o > P.hpos) ? o - 1 : o);
-        dfl d1[2] = {{0.f, 0.f}, {0.f, 0.f}}, d2[2] = {{0.f, 0.f}, {0.f, 0.f}}, da[2] = {{0.f, 0.f}, {0.f, 0.f}};
-        auto term = [&](int k, int h) {
-            const int q = (P.hpos >= 0 && k >= P.hpos) ? k + 1 : k;
-            const float2 dk = oh ? P.hdf[k] : P.ddf[(size_t)k * P.nb + ob], zk = P.z2df[q];
-            const dfl r = dfl_rcp(dfl_add({dk.x, dk.y}, td));  // 1 / (lam - eps_k)
-            const dfl qv = dfl_mul({zk.x, zk.y}, r);
+            const float2 zk = P.z2df[q];
+            const dfl r = dfl_rcp(x);
+            const dfl v = dfl_mul({zk.x, zk.y}, r);
             if (q != o) {
-                d1[h] = dfl_add(d1[h], qv);
-                d2[h] = dfl_add(d2[h], dfl_mul(qv, r));
-                if (ABS) da[h] = dfl_add(da[h], qv.hi < 0.f ? dfl{-qv.hi, -qv.lo} : qv);
+                const dfl w = dfl_mul(v, r);
+                dfl_acc(d1[h], v);
+                dfl_acc(d2[h], w);
+                da += fabsf(v.hi);
+                s3 = fmaf(w.hi, r.hi, s3);
             }
         };
+        const int nk = EV == EV_TWO_DF ? P.nb : M;
         int k = 0;
-        for (; k + 1 < P.nb; k += 2) {
+        for (; k + 1 < nk; k += 2) {
             term(k, 0);
             term(k + 1, 1);
         }
-        if (k < P.nb) term(k, 0);
+        if (k < nk) term(k, 0);
         s1 = (R)dfl_value(dfl_add(d1[0], d1[1]));
         s2 = (R)dfl_value(dfl_add(d2[0], d2[1]));
-        sa = (R)dfl_value(dfl_add(da[0], da[1]));
-        if (P.hpos >= 0 && !oh) {
-            const R r = pole_recip<R>((P.eps[o] - P.hm) + tau);
-            const R qv = P.z2[P.hpos] * r;
-            s1 += qv;
-            s2 = fma(qv, r, s2);
-            if (ABS) sa += fabs(qv);
+        sa = (R)da;
+        if constexpr (EV == EV_TWO_DF)  // the h_- term in R
+            if (P.hpos >= 0 && !oh) {
+                const R r = pole_recip<R>((P.eps[o] - P.hm) + tau);
+                const R qv = P.z2[P.hpos] * r, wv = qv * r;
+                s1 += qv;
+                s2 += wv;
+                sa += fabs(qv);
+                s3 = fmaf((float)wv, (float)r, s3);
+            }
+    } else if constexpr (EV == EV_POLE_F32) {
+        const float tf = (float)tau, po = P.hdf[o].x;
+        float f1 = 0.f, f2 = 0.f, fa = 0.f;
+#pragma unroll 4
+        for (int k = 0; k < M; ++k) {
+            const float r = pole_recip<float>((po - P.hdf[k].x) + tf);
+            const float v = k != o ? P.z2df[k].x * r : 0.f, w = v * r;
+            f1 += v;
+            f2 += w;
+            fa += fabsf(v);
+            s3 = fmaf(w, r, s3);
         }
+        s1 = (R)f1, s2 = (R)f2, sa = (R)fa;
     } else {
         const R eo = P.eps[o];
 #pragma unroll 4
@@ -248,85 +264,122 @@ __device__ __forceinline__ Sec<R> sec_eval(const Poles<R> &P, int o, R tau, R eo
             const R q = P.z2[k] * r;
             if (k != o) {
                 s1 += q;
-                s2 = fma(q, r, s2);
-                if (ABS) sa += fabs(q);
+                if constexpr (sizeof(R) == 4) {
+                    const R w = q * r;
+                    s2 += w;
+                    s3 = fmaf(w, r, s3);
+                    sa += fabs(q);
+                } else {
+                    s2 = fma(q, r, s2);
+                    if (ABS) sa += fabs(q);
+                }
             }
         }
     }
     // origin term: one reciprocal of tau (never zero or subnormal: the
     // iteration keeps it strictly inside its bracket) serves both quotients
     const R rt = pole_recip<R>(tau);
-    const R qo = P.z2[o] * rt;
+    const R qo = P.z2[o] * rt, wo = qo * rt;
     Sec<R> e;
     e.g = (eomh + tau) - s1 - qo;
     e.gp_rest = R(1) + s2;
-    e.gp = e.gp_rest + qo * rt;
+    e.gp = e.gp_rest + wo;
     e.qo = qo;
     e.sabs = sa;
+    e.s3 = fmaf((float)wo, (float)rt, s3);
     return e;
 }
 
-// Fixed-weight iteration for one root in the shifted variable tau about the
-// origin pole o: the origin pole is kept exactly and the rest of g is
-// modelled by one more pole at tau = +D (kind 0) or -D (kind 1), or by a
-// linear term for the two outermost roots (kind 2: below all poles, kind 3:
-// above), matched in value and slope; each model root is safeguarded by the
-// bracket [lo, hi] of sign changes.  On return e is evaluated at tau.
+// One step of the fixed-weight iteration as a correction delta to tau: the
+// origin pole (weight s at distance -tau) is kept exactly and the rest of g
+// is modelled by one more pole at distance -tp (tp = tau -+ D, the other end
+// of the gap; kinds 0 and 1) or by a linear term for the two outermost roots
+// (kind 2: below all poles, kind 3: above), matched in value and slope:
+//   kinds 0, 1: A d^2 + B d + G = 0, A = g + s/tau + ee tp,
+//               B = g (tau + tp) + s tp/tau + ee tp tau, G = g tau tp;
+//   kinds 2, 3: A = ee, B = g + ee tau + s/tau, G = g tau,
+// ee the slope of the rest.  The model root in the gap is the one where the
+// quadratic decreases (kind 3: increases).  A correction needs no more than
+// FP32: its relative error, 10^-6, only enters the next iterate's error
+// (FP64 instructions on this iteration's serial path cost more than they
+// save: a warp's takes 64 cycles of its scheduler's FP64 pipe).
+template <class T>
+__device__ __forceinline__ T sec_step(int kind, T g, T ee, T s, T tau, T tp)
+{
+    const T srt = s * pole_recip<T>(tau);
+    T A, B, G;
+    if (kind <= 1) {
+        A = g + srt + ee * tp;
+        B = g * (tau + tp) + tp * (srt + ee * tau);
+        G = g * tau * tp;
+    } else {
+        A = ee;
+        B = g + ee * tau + srt;
+        G = g * tau;
+    }
+    const T rb = pole_recip<T>(B), a = A * rb, b = G * rb;
+    const T sq = sqrt(fmax(T(1) - T(4) * a * b, T(0)));
+    if ((B < T(0)) != (kind == 3)) return T(-2) * b * pole_recip<T>(T(1) + sq);
+    return (T(1) + sq) * T(-0.5) * pole_recip<T>(a);
+}
+
+// The step at tau, in FP32 where its quantities are inside FP32's range.
+template <class R>
+__device__ __forceinline__ R sec_delta(int kind, const Sec<R> &e, R s, R tau, R D)
+{
+    if constexpr (sizeof(R) == 8) {
+        const float tf = (float)tau, sf = (float)s, ef = (float)e.gp_rest, df = (float)D;
+        if (fabsf(tf) > 1e-18f && sf > 1e-25f && ef < 1e18f)
+            return (R)sec_step<float>(kind, (float)e.g, ef, sf, tf, kind == 0 ? tf - df : tf + df);
+    }
+    return sec_step<R>(kind, e.g, e.gp_rest, s, tau, kind == 0 ? tau - D : tau + D);
+}
+
+// A correction this small against the distance to the nearer end of the gap
+// ends the iteration: tau takes it, and gp its first-order change -2 s3 delta
+// (what is left out is of second order, below the mode's rounding).  FP32:
+// 2^-13; double-float sums: 2^-23; the last FP64 evaluation of a staged
+// solve: 2^-31.
+template <class R>
+__device__ __forceinline__ bool sec_accept(int kind, R D, R limit, R delta, R &tau, Sec<R> &e)
+{
+    const R tp = kind == 0 ? tau - D : tau + D;
+    const R dist = kind <= 1 ? fmin(fabs(tau), fabs(tp)) : fabs(tau);
+    if (!(fabs(delta) <= limit * dist)) return false;
+    e.gp += (R)(-2.0f * e.s3 * (float)delta);
+    tau += delta;
+    return true;
+}
+
+// Safeguarded iteration for one root in the shifted variable tau about the
+// origin pole o; [lo, hi] brackets the sign change.  On return e is evaluated
+// at tau (or corrected to it).
 template <class R, int EV>
 __device__ bool sec_iterate(const Poles<R> &P, R h, int o, int kind, R D, R &lo, R &hi, R &tau,
-                            Sec<R> &e, bool have)
+                            Sec<R> &e, bool have, R ulps = R(8))
 {
     // rounding unit of the sums: 2^-44 covers the double-float sums
-    const R u = (EV == EV_DFLOAT || EV == EV_TWO_DF || EV == EV_NESTED) ? R(5.684341886080802e-14)
-                                                                       : Roundoff<R>::u;
+    constexpr bool kF32 = sizeof(R) == 4 || EV == EV_POLE_F32;
+    // (a stage before another one is run down to its corrections' limit)
+    const R u = ev_is_df(EV) ? R(5.684341886080802e-14) : (kF32 ? R(Roundoff<float>::u) : R(Roundoff<R>::u));
+    const R limit = kF32 ? R(1.2207031e-4) : (ev_is_df(EV) ? R(1.1920929e-7) : R(0));
     const R eomh = P.eps[o] - h;
     const R s = P.z2[o];
     // the non-origin part of the error scale varies slowly with tau (those
     // poles are at least half a gap away): take it from the first evaluation
-    R sa_rest;
-    if (have) {
-        sa_rest = e.sabs;
-    } else {
-        e = sec_eval<R, true, EV>(P, o, tau, eomh);
-        sa_rest = e.sabs;
-        have = true;
-    }
+    if (!have) e = sec_eval<R, true, EV>(P, o, tau, eomh);
+    const R sa_rest = e.sabs;
     for (int it = 0; it < 80; ++it) {
-        if (!have) e = sec_eval<R, false, EV>(P, o, tau, eomh);
-        have = false;
+        if (it) e = sec_eval<R, false, EV>(P, o, tau, eomh);
         e.sabs = sa_rest + fabs(e.qo) + fabs(eomh) + fabs(tau);
-        if (fabs(e.g) <= R(8) * u * e.sabs) return true;
+        if (fabs(e.g) <= ulps * u * e.sabs) return true;
         if (e.g < R(0)) lo = tau;
         else hi = tau;
-        // The quotients below are model-root proposals, safeguarded by the
-        // bracket: reciprocals (pole_recip, within about an ulp) instead of
-        // correctly rounded divisions, which cost several FP64 instructions
-        // each on the iteration's serial path.  A zero or subnormal
-        // denominator gives a non-finite proposal and the bisection step.
-        R tn;
-        const R rt = pole_recip<R>(tau);
-        if (kind <= 1) {
-            // model root of c tau^2 + B tau + s D = 0 in the gap, by the form
-            // without cancellation for the sign of B (B < 0 happens when the
-            // origin pole's weight s is small against the other end's)
-            const R sg = kind == 0 ? R(1) : R(-1);
-            const R tp = tau - sg * D;
-            const R t = e.gp_rest * tp * tp;
-            const R c = sg * (e.g + s * rt + t * pole_recip<R>(tp));
-            const R B = c * D + s + t;
-            const R sq = sqrt(fmax(B * B - R(4) * c * s * D, R(0)));
-            if (B >= R(0) || c == R(0)) tn = sg * R(2) * s * D * pole_recip<R>(B + sq);
-            else tn = sg * (B - sq) * pole_recip<R>(R(2) * c);
-        } else {
-            const R ee = e.gp_rest;
-            const R c = e.g - ee * tau + s * rt;
-            const R sq = sqrt(fmax(c * c + R(4) * ee * s, R(0)));
-            if (kind == 2)
-                tn = (c >= R(0)) ? (-c - sq) * pole_recip<R>(R(2) * ee) : -R(2) * s * pole_recip<R>(sq - c);
-            else
-                tn = (c <= R(0)) ? (sq - c) * pole_recip<R>(R(2) * ee) : R(2) * s * pole_recip<R>(c + sq);
-        }
-        if (!(tn > lo && tn < hi)) tn = R(0.5) * (lo + hi);
+        const R delta = sec_delta<R>(kind, e, s, tau, D);
+        R tn = tau + delta;
+        const bool in = tn > lo && tn < hi;
+        if (limit > R(0) && in && sec_accept<R>(kind, D, limit, delta, tau, e)) return true;
+        if (!in) tn = R(0.5) * (lo + hi);
         const bool tiny = fabs(tn - tau) <= R(2) * u * fabs(tn);
         tau = tn;
         if (tiny) {
@@ -345,8 +398,14 @@ __device__ bool sec_iterate(const Poles<R> &P, R h, int o, int kind, R D, R &lo,
 // `guess`, which lies in the same gap): origin = pole nearer the guess,
 // bracket = the whole gap, started at the guess; if the root ends in the
 // far half of the gap it is refined once more about the other pole.
-// EV: how the secular sums are formed (see sec_eval).
-template <class R, int EV = EV_PLAIN>
+// EV: how the final sums are formed (see sec_eval).  EVP, EV0 (R = double):
+// cheaper sums for a staged solve -- the iteration runs with EV0 (cold
+// starts only), then EVP, to their own accuracy, and EV evaluates once more
+// and corrects: an FP64 term costs about 450 cycles of a scheduler (7
+// instructions at 64 cycles a warp), a double-float one 55 and an FP32 one
+// 12.  Where the correction is not small (a root so close to its pole or so
+// sensitive that the stage before could not resolve it) EV iterates.
+template <class R, int EV = EV_PLAIN, int EVP = EV, int EV0 = EVP>
 __device__ void secular_root(int r, const Poles<R> &P, R h, R Z2, bool warm, R guess, R &lam, R &q0,
                              uint32_t &st, int *o_out = nullptr, R *tau_out = nullptr)
 {
@@ -355,32 +414,37 @@ __device__ void secular_root(int r, const Poles<R> &P, R h, R Z2, bool warm, R g
     int o, kind;
     R lo, hi, D = 0, tau;
     Sec<R> e;
-    bool have = false, conv;
+    bool have = false, conv, cold = true;
     if (r > 0 && r < M) {
         const int L = r - 1;
         D = eps[r] - eps[L];
         if (warm && guess > eps[L] && guess < eps[r]) {
+            cold = false;
             if (guess - eps[L] <= eps[r] - guess) {
                 o = L; kind = 0; lo = 0; hi = D; tau = guess - eps[L];
             } else {
                 o = r; kind = 1; lo = -D; hi = 0; tau = guess - eps[r];
             }
-            conv = sec_iterate<R, EV>(P, h, o, kind, D, lo, hi, tau, e, false);
-            if (kind == 0 && tau > R(0.5) * D) {
-                o = r; kind = 1; lo = fmin(lo - D, -R(0.5) * D); hi = 0; tau = tau - D;
-                conv = sec_iterate<R, EV>(P, h, o, kind, D, lo, hi, tau, e, false);
-            } else if (kind == 1 && tau < -R(0.5) * D) {
-                o = L; kind = 0; lo = 0; hi = fmax(hi + D, R(0.5) * D); tau = tau + D;
-                conv = sec_iterate<R, EV>(P, h, o, kind, D, lo, hi, tau, e, false);
-            }
         } else {
-            const Sec<R> em = sec_eval<R, true, EV>(P, L, R(0.5) * D, eps[L] - h);
-            if (em.g >= R(0)) {
-                o = L; kind = 0; lo = 0; hi = R(0.5) * D; tau = R(0.5) * D; e = em; have = true;
+            e = sec_eval<R, true, EV0>(P, L, R(0.5) * D, eps[L] - h);
+            have = true;
+            if (e.g >= R(0)) {
+                o = L; kind = 0; lo = 0; hi = R(0.5) * D; tau = R(0.5) * D;
             } else {
+                // the same sums about the other pole: the two ends' terms
+                // change places
                 o = r; kind = 1; lo = -R(0.5) * D; hi = 0; tau = -R(0.5) * D;
+                const R rd = pole_recip<R>(tau), qr = P.z2[r] * rd, qL = e.qo;
+                e.gp_rest += (e.gp - e.gp_rest) - qr * rd;
+                e.sabs += fabs(qL) - fabs(qr);
+                e.qo = qr;
             }
-            conv = sec_iterate<R, EV>(P, h, o, kind, D, lo, hi, tau, e, have);
+            // coarser sums may misjudge a root near the middle: the later
+            // stages get the whole gap
+            if constexpr (EV0 != EV) {
+                lo = kind == 0 ? R(0) : -D;
+                hi = kind == 0 ? D : R(0);
+            }
         }
     } else {
         if (r == 0) {
@@ -400,13 +464,50 @@ __device__ void secular_root(int r, const Poles<R> &P, R h, R Z2, bool warm, R g
         }
         if (warm) {
             const R tg = guess - eps[o];
-            if (tg > lo && tg < hi) tau = tg;
+            if (tg > lo && tg < hi) {
+                tau = tg;
+                cold = false;
+            }
         }
-        conv = sec_iterate<R, EV>(P, h, o, kind, D, lo, hi, tau, e, false);
+    }
+    // the bracket of a stage with coarser sums is its own: a sign decided by
+    // rounding must not shut the root out of the next stage's
+    if constexpr (EV0 != EVP)
+        if (cold) {
+            R l0 = lo, h0 = hi;
+            sec_iterate<R, EV0>(P, h, o, kind, D, l0, h0, tau, e, have);
+            have = false;
+        }
+    R lp = lo, hp = hi;
+    constexpr R ulps = EVP == EV ? R(8) : R(0.25);
+    conv = sec_iterate<R, EVP>(P, h, o, kind, D, lp, hp, tau, e, have, ulps);
+    if constexpr (EVP == EV) lo = lp, hi = hp;
+    if (!cold && kind <= 1) {
+        bool moved = false;
+        if (kind == 0 && tau > R(0.5) * D) {
+            o = r; kind = 1; lo = fmin(lo - D, -R(0.5) * D); hi = 0; tau = tau - D;
+            moved = true;
+        } else if (kind == 1 && tau < -R(0.5) * D) {
+            o = r - 1; kind = 0; lo = 0; hi = fmax(hi + D, R(0.5) * D); tau = tau + D;
+            moved = true;
+        }
+        if (moved) {
+            lp = lo, hp = hi;
+            conv = sec_iterate<R, EVP>(P, h, o, kind, D, lp, hp, tau, e, false, ulps);
+        }
+    }
+    if constexpr (EVP != EV) {
+        const float s3 = e.s3;
+        e = sec_eval<R, false, EV>(P, o, tau, eps[o] - h);
+        e.s3 = s3;
+        const R delta = sec_delta<R>(kind, e, P.z2[o], tau, D);
+        if (!(conv && tau + delta > lo && tau + delta < hi && sec_accept<R>(kind, D, R(4.656612873077393e-10), delta, tau, e)))
+            conv = sec_iterate<R, EV>(P, h, o, kind, D, lo, hi, tau, e, false);
     }
     if (!conv) st |= ST_SECULAR;
     lam = eps[o] + tau;
-    q0 = R(1) / sqrt(e.gp);
+    if constexpr (sizeof(R) == 4) q0 = R(1) / sqrt(e.gp);
+    else q0 = rsqrt(e.gp);
     if (o_out) *o_out = o;  // lam = eps[o] + tau with tau exact
     if (tau_out) *tau_out = tau;
 }

@@ -51,7 +51,9 @@ __device__ __forceinline__ void slot_tree_sum(double *red, int r, bool inslot, i
 // mode 0: eigenpairs and force at the stored position (cold start);
 // mode 1: full first half of a step (kick, drift, eigenpairs, force, kick).
 // tpb trajectories per CTA, one thread per root.
-// DF: the secular sums in double-float arithmetic (mixed path).
+// The secular iteration runs on double-float sums (FP32 pipe); DF (mixed
+// path): they are the result's too, else one FP64 evaluation at the end
+// corrects root and slope (secular_root).
 template <bool DF>
 __global__ void __launch_bounds__(256, 3) k_eigen(DevState s, ModelDev md, double dt, int mode, int tpb)
 {
@@ -63,12 +65,12 @@ __global__ void __launch_bounds__(256, 3) k_eigen(DevState s, ModelDev md, doubl
     const bool act = t >= 0 && !(s.status[t] & ST_DONE);
     const int P = eigen_pow2(N);                         // reduction width
     double *eps_s = sh;                                  // [M], shared by the slots
-    const int per = M + 2 * N + P + (DF ? M : 0);
+    const int per = 2 * M + 2 * N + P;
     double *z2_s = eps_s + M + (slot < tpb ? slot : 0) * per;  // [M]
     double *lam_s = z2_s + M;                            // [N]
     double *q0_s = lam_s + N;                            // [N]
     double *red_s = q0_s + N;                            // [P] slot reductions
-    float2 *z2df_s = reinterpret_cast<float2 *>(red_s + P);  // [M] z_k^2 as double-float (DF)
+    float2 *z2df_s = reinterpret_cast<float2 *>(red_s + P);  // [M] z_k^2 as double-float
     const bool inslot = slot < tpb;
     for (int k = threadIdx.x; k < M; k += blockDim.x) eps_s[k] = s.eps[k];
     double x = 0.0, p = 0.0, guess = 0.0;
@@ -98,10 +100,8 @@ __global__ void __launch_bounds__(256, 3) k_eigen(DevState s, ModelDev md, doubl
         for (int k = r; k < M; k += N) {
             const double z = s.z0[k] * mv.f;
             z2_s[k] = z * z;
-            if (DF) {
-                const dfl zd = dfl_from(z * z);
-                z2df_s[k] = make_float2(zd.hi, zd.lo);
-            }
+            const dfl zd = dfl_from(z * z);
+            z2df_s[k] = make_float2(zd.hi, zd.lo);
         }
     }
     __syncthreads();
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(256, 3) k_eigen(DevState s, ModelDev md, doubl
             if (DF)
                 secular_root<double, EV_DFLOAT>(r, pp, mv.h, Z2, mode == 1, guess, l, q, st, &ro_r, &rt_r);
             else
-                secular_root<double, EV_TABLE>(r, pp, mv.h, Z2, mode == 1, guess, l, q, st, &ro_r, &rt_r);
+                secular_root<double, EV_TABLE, EV_DFLOAT>(r, pp, mv.h, Z2, mode == 1, guess, l, q, st, &ro_r, &rt_r);
         } else {
             // no coupling: the eigenvalues are h and the bath energies
             int pos = 0;
@@ -1546,7 +1546,7 @@ cudaError_t launch_eigen(const DevState &s, const ModelDev &md, double dt, int m
     const int threads = round32(tpb * s.N);
     const bool df = s.eigen_dfloat != 0;
     const size_t smem =
-        (size_t)(s.M + tpb * (s.M + 2 * s.N + eigen_pow2(s.N) + (df ? s.M : 0))) * sizeof(double);
+        (size_t)(s.M + tpb * (2 * s.M + 2 * s.N + eigen_pow2(s.N))) * sizeof(double);
     if (df) k_eigen<true><<<(unsigned)((s.n + tpb - 1) / tpb), threads, smem, st>>>(s, md, dt, mode, tpb);
     else k_eigen<false><<<(unsigned)((s.n + tpb - 1) / tpb), threads, smem, st>>>(s, md, dt, mode, tpb);
     return cudaGetLastError();

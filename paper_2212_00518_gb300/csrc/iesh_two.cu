@@ -214,9 +214,10 @@ struct Eig2Slot {
 // mode 0: eigenpairs and forces at x (state set-up).  mode 1: a step's
 // kick + drift, eigenpairs at the new x, forces and the second kick.
 // tpb trajectories per CTA (slots of N threads), one thread per root; every
-// barrier is reached by all threads of the CTA.  DF: the secular sums over
-// the bath poles in double-float arithmetic (mixed path; the bath
-// differences from the context's table, those to h_- per trajectory).
+// barrier is reached by all threads of the CTA.  The secular iteration runs
+// on double-float sums over the bath poles (the bath differences from the
+// context's table, those to h_- per trajectory); DF (mixed path): they are
+// the result's too, else one FP64 evaluation at the end corrects it.
 template <bool DF>
 __global__ void __launch_bounds__(256, 3) k2_eigen(DevState s, Model2Dev md, double dt, int mode, int tpb)
 {
@@ -228,18 +229,22 @@ __global__ void __launch_bounds__(256, 3) k2_eigen(DevState s, Model2Dev md, dou
     const int64_t t = inslot ? traj_of(s, (int64_t)blockIdx.x * tpb + slot) : -1;
     const bool act = t >= 0 && !(s.status[t] & ST_DONE);
     const int Pw = eigen_pow2(N);                          // reduction width
-    const int per = 2 * (M + 1) + 3 * N + 4 * Pw + (DF ? 2 * M + 1 : 0);
+    const int per = 2 * (M + 1) + 3 * N + 4 * Pw + 2 * M + 1;
     double *eps_s = e2_sh;                                 // [M] bath energies, shared
-    double *pole = eps_s + M + (inslot ? slot : 0) * per;  // [M + 1] sorted poles
+    float2 *ew_s = reinterpret_cast<float2 *>(eps_s + M);  // [M] (eps_k, w_k) in FP32, shared
+    double *pole = eps_s + 2 * M + (inslot ? slot : 0) * per;  // [M + 1] sorted poles
     double *wt = pole + (M + 1);                           // [M + 1] their weights
     double *lam_s = wt + (M + 1);                          // [N]
     double *Q0_s = lam_s + N;                              // [N]
     double *Q1_s = Q0_s + N;                               // [N]
     double *red = Q1_s + N;                                // [4][Pw] reductions / staging
-    float2 *z2df = reinterpret_cast<float2 *>(red + 4 * Pw);  // [M + 1] weights as double-float (DF)
-    float2 *hdf = z2df + (M + 1);                          // [M] h_- - eps_k as double-float (DF)
-    Eig2Slot *sl = reinterpret_cast<Eig2Slot *>(e2_sh + M + tpb * per) + (inslot ? slot : 0);
-    for (int k = threadIdx.x; k < M; k += blockDim.x) eps_s[k] = s.eps[k];
+    float2 *z2df = reinterpret_cast<float2 *>(red + 4 * Pw);  // [M + 1] weights as double-float
+    float2 *hdf = z2df + (M + 1);                          // [M] h_- - eps_k as double-float
+    Eig2Slot *sl = reinterpret_cast<Eig2Slot *>(e2_sh + 2 * M + tpb * per) + (inslot ? slot : 0);
+    for (int k = threadIdx.x; k < M; k += blockDim.x) {
+        eps_s[k] = s.eps[k];
+        ew_s[k] = make_float2((float)s.eps[k], (float)(s.z0[k] * s.z0[k]));
+    }
     // warm start: the previous roots extrapolated linearly (each thread reads
     // its own entries before it overwrites them)
     double guess = 0.0, lam_old = 0.0;
@@ -301,22 +306,18 @@ __global__ void __launch_bounds__(256, 3) k2_eigen(DevState s, Model2Dev md, dou
             const double w = (c0 * c0 + c1 * c1) * (s.z0[k] * s.z0[k]);
             pole[q] = eps_s[k];
             wt[q] = w;
-            if (DF) {
-                const dfl wd = dfl_from(w);
-                z2df[q] = make_float2(wd.hi, wd.lo);
-                if (cs == 0) {
-                    const dfl hd = dfl_from(hm - eps_s[k]);
-                    hdf[k] = make_float2(hd.hi, hd.lo);
-                }
+            const dfl wd = dfl_from(w);
+            z2df[q] = make_float2(wd.hi, wd.lo);
+            if (cs == 0) {
+                const dfl hd = dfl_from(hm - eps_s[k]);
+                hdf[k] = make_float2(hd.hi, hd.lo);
             }
         }
         if (cs == 0 && r == 0) {
             pole[pos] = hm;
             wt[pos] = tt * tt;
-            if (DF) {
-                const dfl wd = dfl_from(tt * tt);
-                z2df[pos] = make_float2(wd.hi, wd.lo);
-            }
+            const dfl wd = dfl_from(tt * tt);
+            z2df[pos] = make_float2(wd.hi, wd.lo);
         }
     }
     __syncthreads();
@@ -357,13 +358,9 @@ __global__ void __launch_bounds__(256, 3) k2_eigen(DevState s, Model2Dev md, dou
                 // an extrapolation outside the root's pole gap falls back to the last root
                 const double glo = r > 0 ? pole[r - 1] : -INFINITY, ghi = r < P ? pole[r] : INFINITY;
                 if (!(guess > glo && guess < ghi)) guess = lam_old;
-                if (DF) {
-                    const Poles<double> pp = {P, pole, wt, nullptr, s.poledf, z2df, M, cs == 0 ? pos : -1, hm, hdf};
-                    secular_root<double, EV_TWO_DF>(r, pp, sl->hp, Z2, mode == 1, guess, lam, qp, st, &o, &tau);
-                } else {
-                    const Poles<double> pp = {P, pole, wt, nullptr, nullptr, nullptr};
-                    secular_root<double>(r, pp, sl->hp, Z2, mode == 1, guess, lam, qp, st, &o, &tau);
-                }
+                const Poles<double> pp = {P, pole, wt, nullptr, s.poledf, z2df, M, cs == 0 ? pos : -1, hm, hdf};
+                if (DF) secular_root<double, EV_TWO_DF>(r, pp, sl->hp, Z2, mode == 1, guess, lam, qp, st, &o, &tau);
+                else secular_root<double, EV_PLAIN, EV_TWO_DF>(r, pp, sl->hp, Z2, mode == 1, guess, lam, qp, st, &o, &tau);
                 if (cs == 0) {
                     // lam - h_-: the exact offset when the origin pole is h_- itself
                     const double lmh = (o == pos) ? tau : (pole[o] - hm) + tau;
@@ -411,10 +408,10 @@ __global__ void __launch_bounds__(256, 3) k2_eigen(DevState s, Model2Dev md, dou
         const float ljf = (float)lj, lpf = (float)lp;
         float acc = 0.0f;
         for (int k = 0; k < M; ++k) {
-            const float ek = (float)eps_s[k];
-            const float den = (ljf - ek) * (lpf - ek);
-            const float w = (float)(s.z0[k] * s.z0[k]);
-            if (den != 0.0f) acc += __fdividef(w, den);
+            // FP32 copies: a conversion in the loop costs an FP64 instruction
+            const float2 ew = ew_s[k];
+            const float den = (ljf - ew.x) * (lpf - ew.x);
+            if (den != 0.0f) acc += __fdividef(ew.y, den);
         }
         const float ov = (float)(q0 * p0 + q1 * p1) + Aj * Ap * acc;
         if (ov <= -0.5f) {
@@ -1075,10 +1072,21 @@ size_t dense_reduce_smem(int N)
 }
 
 // Shared memory of k2_eigen with tpb slots.
-size_t eigen2_smem(int N, int M, int tpb, bool df)
+size_t eigen2_smem(int N, int M, int tpb)
 {
-    const int per = 2 * (M + 1) + 3 * N + 4 * eigen_pow2(N) + (df ? 2 * M + 1 : 0);
-    return (size_t)(M + tpb * per) * sizeof(double) + (size_t)tpb * sizeof(Eig2Slot);
+    const int per = 2 * (M + 1) + 3 * N + 4 * eigen_pow2(N) + 2 * M + 1;
+    return (size_t)(2 * M + tpb * per) * sizeof(double) + (size_t)tpb * sizeof(Eig2Slot);
+}
+
+// The shared-memory limit is a process-wide function attribute: only raised.
+template <class F>
+cudaError_t raise_smem(F *fn, size_t bytes)
+{
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, fn);
+    if (e == cudaSuccess && fa.maxDynamicSharedSizeBytes < (int)bytes)
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return e;
 }
 
 }  // namespace
@@ -1173,7 +1181,7 @@ cudaError_t launch_eigen2(iesh2_ctx *ctx, double dt, int mode)
     const int tpb = eigen_tpb(d.N);
     const int threads = (tpb * d.N + 31) & ~31;
     const unsigned blocks = (unsigned)((d.n + tpb - 1) / tpb);
-    const size_t smem = eigen2_smem(d.N, d.M, tpb, ctx->mixed);
+    const size_t smem = eigen2_smem(d.N, d.M, tpb);
     if (ctx->mixed) k2_eigen<true><<<blocks, threads, smem, ctx->stream>>>(d, ctx->md, dt, mode, tpb);
     else k2_eigen<false><<<blocks, threads, smem, ctx->stream>>>(d, ctx->md, dt, mode, tpb);
     return cudaGetLastError();
@@ -1314,7 +1322,7 @@ iesh_status iesh2_create(iesh2_ctx **out, const iesh2_model *model, int precisio
     if (ctx->nested && ctx->mixed) A2(ppdf_d, (size_t)M)
     A2(eps_d, (size_t)M) A2(sq_d, (size_t)M) A2(prof_d, (size_t)2 * M)
     float2 *poledf = nullptr;
-    if (ctx->mixed) A2(poledf, (size_t)M * M)
+    A2(poledf, (size_t)M * M)
 #undef A2
     d.C = Cd;
     d.eps = eps_d;
@@ -1326,10 +1334,8 @@ iesh_status iesh2_create(iesh2_ctx **out, const iesh2_model *model, int precisio
     configure_cheb_tc16();
     configure_cheb_fx();
     // the slots of the eigen kernel can pass the 48 KiB default (N near 65)
-    CU2(cudaFuncSetAttribute(k2_eigen<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)eigen2_smem(N, M, eigen_tpb(N), false)));
-    CU2(cudaFuncSetAttribute(k2_eigen<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)eigen2_smem(N, M, eigen_tpb(N), true)));
+    CU2(raise_smem(k2_eigen<false>, eigen2_smem(N, M, eigen_tpb(N))));
+    CU2(raise_smem(k2_eigen<true>, eigen2_smem(N, M, eigen_tpb(N))));
     CU2(cudaMemcpyAsync(eps_d, eps.data(), M * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
     CU2(cudaMemcpyAsync(sq_d, sq.data(), M * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
     // coupling profiles of the dense path: sqrt(w_k), times the Lorentzian
@@ -1360,18 +1366,15 @@ iesh_status iesh2_create(iesh2_ctx **out, const iesh2_model *model, int precisio
             CU2(cudaFuncSetAttribute(k2g_reduce, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)(kDenseSmemCap + 2048)));
     }
-    std::vector<float2> pf;
-    if (ctx->mixed) {
-        // bath pole differences eps_o - eps_k as double-float pairs, [k][o]
-        pf.resize((size_t)M * M);
-        for (int kk = 0; kk < M; ++kk)
-            for (int o = 0; o < M; ++o) {
-                const double v = eps[o] - eps[kk];
-                const float hi = (float)v;
-                pf[(size_t)kk * M + o] = make_float2(hi, (float)(v - (double)hi));
-            }
-        CU2(cudaMemcpyAsync(poledf, pf.data(), pf.size() * sizeof(float2), cudaMemcpyHostToDevice, ctx->stream));
-    }
+    // bath pole differences eps_o - eps_k as double-float pairs, [k][o]
+    std::vector<float2> pf((size_t)M * M);
+    for (int kk = 0; kk < M; ++kk)
+        for (int o = 0; o < M; ++o) {
+            const double v = eps[o] - eps[kk];
+            const float hi = (float)v;
+            pf[(size_t)kk * M + o] = make_float2(hi, (float)(v - (double)hi));
+        }
+    CU2(cudaMemcpyAsync(poledf, pf.data(), pf.size() * sizeof(float2), cudaMemcpyHostToDevice, ctx->stream));
     std::vector<float2> ppf;
     if (ppdf_d) {
         // prof_0k prof_1k as double-float pairs (the nested path's couplings)
