@@ -69,6 +69,88 @@ __device__ __forceinline__ int pivot_key(float2 v)  // max(|re|, |im|), monotoni
 }
 
 
+// The chosen hop (slot s_hop_a to orbital s_hop_m; s_hop_a < 0: none) of the
+// one-coordinate model: the energy-conserving rescale, the force on the new
+// surface, counters, the finished test and the population records.  All
+// threads of the CTA call it after a barrier; occ_s is shared, red too.
+template <class CT>
+__device__ __forceinline__ void hop_apply(const DevState &s, int64_t t, double mass, double *red, int *occ_s, double geo_h,
+                                          double geo_dh, double geo_k, int s_hop_a, int s_hop_m, const CT *Ct)
+{
+    const int N = s.N, Ne = s.Ne;
+    const double *lam_s = s.lam + t * N, *q0_s = s.q0 + t * N;
+    // ---- hop, rescale, force, counters (thread 0)
+    if (threadIdx.x == 0) {
+        double p = s.p[t];
+        if (s_hop_a >= 0) {
+            const int a = s_hop_a, m = s_hop_m;
+            const double dE = lam_s[m] - lam_s[occ_s[a]];
+            const double p2 = p * p - 2.0 * mass * dE;
+            if (p2 >= 0.0) {
+                p = (p >= 0.0 ? 1.0 : -1.0) * sqrt(p2);
+                // replace s_a by m and keep the list sorted
+                int b = a;
+                occ_s[b] = m;
+                while (b > 0 && occ_s[b - 1] > occ_s[b]) {
+                    const int tmp = occ_s[b - 1];
+                    occ_s[b - 1] = occ_s[b];
+                    occ_s[b] = tmp;
+                    --b;
+                }
+                while (b < Ne - 1 && occ_s[b + 1] < occ_s[b]) {
+                    const int tmp = occ_s[b + 1];
+                    occ_s[b + 1] = occ_s[b];
+                    occ_s[b] = tmp;
+                    ++b;
+                }
+                for (int q = 0; q < Ne; ++q) s.occ[t * Ne + q] = (int16_t)occ_s[q];
+                double F = -s.dU0[t];
+                for (int q = 0; q < Ne; ++q) {
+                    const int i = occ_s[q];
+                    F -= q0_s[i] * q0_s[i] * (geo_dh + 2.0 * geo_k * (lam_s[i] - geo_h));
+                }
+                s.F[t] = F;
+                s.p[t] = p;
+                s.hops[t] += 1;
+            } else {
+                s.frus[t] += 1;
+            }
+        }
+        s.vprev[t] = p / mass;
+        const int64_t ns = s.nstep[t] + 1;
+        s.nstep[t] = ns;
+        if (s.z_done > 0.0 && s.x[t] > s.z_done) atomicOr(&s.status[t], ST_DONE);
+    }
+    // ---- observables
+    if (s.record_every > 0) {
+        __syncthreads();
+        const int64_t ns = s.nstep[t];
+        if (ns % s.record_every == 0) {
+            const int64_t r = ns / s.record_every - 1;
+            if (r < s.max_records) {
+                double psh = 0.0, pwf = 0.0;
+                for (int a = threadIdx.x; a < Ne; a += blockDim.x) {
+                    const double q = q0_s[occ_s[a]];
+                    psh += q * q;
+                    double ar = 0.0, ai = 0.0;
+                    for (int i = 0; i < N; ++i) {
+                        const double2 cv = to_d2(Ct[(int64_t)a * N + i]);
+                        ar = fma(q0_s[i], cv.x, ar);
+                        ai = fma(q0_s[i], cv.y, ai);
+                    }
+                    pwf += ar * ar + ai * ai;
+                }
+                psh = block_sum(psh, red);
+                pwf = block_sum(pwf, red);
+                if (threadIdx.x == 0) {
+                    s.rec_sh[r * s.n + t] = psh;
+                    s.rec_wf[r * s.n + t] = pwf;
+                }
+            }
+        }
+    }
+}
+
 // After the hop probabilities G[a][m] (slot a, orbital m; FP64, written and
 // followed by a barrier): the selection with one uniform zeta in the order
 // (slot a ascending, m ascending), then either the hand-over of the chosen
@@ -155,76 +237,7 @@ __device__ __forceinline__ void hop_finish(const DevState &s, int64_t t, double 
         if (threadIdx.x == 0) s.hop_pair[t] = s_hop_a >= 0 ? s_hop_a * N + s_hop_m : -1;
         return;
     }
-    // ---- hop, rescale, force, counters (thread 0)
-    if (threadIdx.x == 0) {
-        double p = s.p[t];
-        if (s_hop_a >= 0) {
-            const int a = s_hop_a, m = s_hop_m;
-            const double dE = lam_s[m] - lam_s[occ_s[a]];
-            const double p2 = p * p - 2.0 * mass * dE;
-            if (p2 >= 0.0) {
-                p = (p >= 0.0 ? 1.0 : -1.0) * sqrt(p2);
-                // replace s_a by m and keep the list sorted
-                int b = a;
-                occ_s[b] = m;
-                while (b > 0 && occ_s[b - 1] > occ_s[b]) {
-                    const int tmp = occ_s[b - 1];
-                    occ_s[b - 1] = occ_s[b];
-                    occ_s[b] = tmp;
-                    --b;
-                }
-                while (b < Ne - 1 && occ_s[b + 1] < occ_s[b]) {
-                    const int tmp = occ_s[b + 1];
-                    occ_s[b + 1] = occ_s[b];
-                    occ_s[b] = tmp;
-                    ++b;
-                }
-                for (int q = 0; q < Ne; ++q) s.occ[t * Ne + q] = (int16_t)occ_s[q];
-                double F = -s.dU0[t];
-                for (int q = 0; q < Ne; ++q) {
-                    const int i = occ_s[q];
-                    F -= q0_s[i] * q0_s[i] * (geo_dh + 2.0 * geo_k * (lam_s[i] - geo_h));
-                }
-                s.F[t] = F;
-                s.p[t] = p;
-                s.hops[t] += 1;
-            } else {
-                s.frus[t] += 1;
-            }
-        }
-        s.vprev[t] = p / mass;
-        const int64_t ns = s.nstep[t] + 1;
-        s.nstep[t] = ns;
-        if (s.z_done > 0.0 && s.x[t] > s.z_done) atomicOr(&s.status[t], ST_DONE);
-    }
-    // ---- observables
-    if (s.record_every > 0) {
-        __syncthreads();
-        const int64_t ns = s.nstep[t];
-        if (ns % s.record_every == 0) {
-            const int64_t r = ns / s.record_every - 1;
-            if (r < s.max_records) {
-                double psh = 0.0, pwf = 0.0;
-                for (int a = threadIdx.x; a < Ne; a += blockDim.x) {
-                    const double q = q0_s[occ_s[a]];
-                    psh += q * q;
-                    double ar = 0.0, ai = 0.0;
-                    for (int i = 0; i < N; ++i) {
-                        const double2 cv = to_d2(Ct[(int64_t)a * N + i]);
-                        ar = fma(q0_s[i], cv.x, ar);
-                        ai = fma(q0_s[i], cv.y, ai);
-                    }
-                    pwf += ar * ar + ai * ai;
-                }
-                psh = block_sum(psh, red);
-                pwf = block_sum(pwf, red);
-                if (threadIdx.x == 0) {
-                    s.rec_sh[r * s.n + t] = psh;
-                    s.rec_wf[r * s.n + t] = pwf;
-                }
-            }
-        }
-    }
+    hop_apply<CT>(s, t, mass, red, occ_s, geo_h, geo_dh, geo_k, s_hop_a, s_hop_m, Ct);
 }
 
 }  // namespace iesh

@@ -1699,6 +1699,7 @@ void configure_hop_smem()
     allow_max_smem(k_hop<float2, 256, 4, true>);
     allow_max_smem(k_cheb_f32t<4, 1>);
     allow_max_smem(k_cheb_f32t<4, 2>);
+    configure_hop_bj();
     configure_hop_gjl();
 }
 
@@ -1706,8 +1707,10 @@ cudaError_t launch_hop(const DevState &s, double dt, double mass, uint64_t seed,
                        double *g_out, cudaStream_t st, bool mixed, bool ext)
 {
     if (s.n == 0) return cudaSuccess;
-    // mixed path: the register-resident Gauss-Jordan kernel where it fits,
-    // unless a hop CTA size was requested
+    // mixed path: Gauss-Jordan, blocked for small matrices, else slot by slot in
+    // registers where it fits, unless a hop CTA size was requested
+    if (mixed && s.hop_threads == 0 && hop_bj_eligible(s.N, s.Ne))
+        return launch_hop_bj(s, dt, mass, seed, g_out, st, ext);
     if (mixed && s.hop_threads == 0 && hop_gj_eligible(s.N, s.Ne))
         return launch_hop_gj(s, dt, mass, seed, g_out, st, ext);
     if (mixed && s.hop_threads == 0 && hop_gjl_eligible(s.N, s.Ne))
