@@ -297,20 +297,25 @@ iesh_status iesh_ensemble_destroy(iesh_ensemble *ens);
 const char *iesh_ensemble_last_error(const iesh_ensemble *ens);
 
 /* Kernel shapes.  FP64 contexts: cheb_ept (1 or 2) electrons per thread and
- * cheb_G column groups per CTA of the propagator (cheb_G * N <= 1024).
+ * cheb_G column groups per CTA of the propagator (cheb_G * N <= 1024); from
+ * N = 28 (and N * Ne = 392) the propagator runs on the tensor cores and takes
+ * cheb_ept * cheb_G as the electrons of a block, at most its built-in width.
  * Mixed contexts: cheb_ept 4 (each thread holds 4 orbitals x 4 electrons,
  * two CTAs per SM) with cheb_G * ceil(N/4) <= 256 and 8 * Np * (8 cheb_G +
  * 1) + 192 * Np bytes of shared memory (Np = N rounded up to a multiple of
  * 4; the second term stages W) at most 110 KiB; or cheb_ept 32 (8 orbitals
  * x 4 electrons per thread, one CTA per SM) with cheb_G * ceil(ceil(N/4)/2)
- * <= 256 and the same shared memory at most 220 KiB; or cheb_ept 8 with
+ * <= 256 and the same shared memory at most 220 KiB (with 128 < N and Ne >=
+ * 16, or N >= 192 and Ne >= 6, both name the tensor-core kernel for two row
+ * tiles, with 4 cheb_G electrons per block, at most 16); or cheb_ept 8 with
  * cheb_G 1, the tensor-core kernel (N <= 128, Ne <= 56, 3xTF32); or
  * cheb_ept 16 with cheb_G 1, the tensor-core kernel on FP16 split operands
  * with two CTAs per SM (N <= 128, Ne <= 56, its shared memory at most 110
  * KiB).  hop_threads (256 or 512):
  * threads of the LU hop kernel; 0 restores the built-in choice, which for
  * mixed contexts is a Gauss-Jordan elimination of all determinant ratios,
- * in registers for N <= 128 and Ne <= 56 and with the rows past 128 in
+ * in blocks of four for N <= 96 and Ne <= 48, slot by slot in registers for
+ * N <= 128 and Ne <= 56 and with the rows past 128 in
  * shared memory up to N = 256, Ne = 112 (the skip bound saves no work
  * there and is not applied; its FP32 ratios round differently from the
  * LU's, about 1e-7 relative); IESH_EINVAL otherwise.  The propagator shapes do not change results

@@ -385,6 +385,10 @@ iesh_status iesh_create(iesh_ctx **out, const iesh_model *model, const iesh_opti
         d.fx_work_bytes = cheb_fx_work_bytes(N, Ne, max_traj);
         A(d.fx_work, d.fx_work_bytes)
     }
+    if (ctx->mixed && cheb_tcl_eligible(N, Ne)) {
+        d.fx_work_bytes = cheb_tcl_work_bytes(N, Ne, max_traj);
+        A(d.fx_work, d.fx_work_bytes)
+    }
     A(ctx->live, T)
     A(ctx->n_live, 1)
     A(ctx->obs, 4 * T)
@@ -413,6 +417,7 @@ iesh_status iesh_create(iesh_ctx **out, const iesh_model *model, const iesh_opti
     configure_cheb_tc();
     configure_cheb_tc16();
     configure_cheb_fx();
+    configure_cheb_tcl();
     {
         std::vector<float> ed((size_t)M * M);
         for (int a = 0; a < M; ++a)

@@ -77,6 +77,12 @@ bool cheb_fx_eligible(int N, int Ne);
 size_t cheb_fx_work_bytes(int N, int Ne, int64_t max_traj);
 void configure_cheb_fx();
 cudaError_t launch_cheb_fx(const DevState &s, double dt, cudaStream_t st);
+// mixed-path propagator on the tensor cores for 128 < N <= 256 (FP32 numbers
+// as FP16 digits); its workspace is made with the context
+bool cheb_tcl_eligible(int N, int Ne);
+size_t cheb_tcl_work_bytes(int N, int Ne, int64_t max_traj);
+void configure_cheb_tcl();
+cudaError_t launch_cheb_tcl(const DevState &s, double dt, cudaStream_t st);
 // unitarity check of the coefficient columns (sets ST_NORM), observables
 // out[4][n] = (kinetic energy, potential energy, occupied-surface and
 // wavefunction impurity populations), batch status summary out[9]

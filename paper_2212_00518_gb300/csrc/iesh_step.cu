@@ -1621,8 +1621,9 @@ cudaError_t launch_cheb(const DevState &s, double dt, bool mixed, cudaStream_t s
 {
     if (s.n == 0) return cudaSuccess;
     if (mixed) {
-        // tensor cores (3xTF32) when the trajectory fits one CTA, unless a
-        // SIMT shape was requested
+        // N > 128: tensor cores with FP32 digits (any requested shape sets its
+        // blocks' width; the bits are the same)
+        if (s.fx_work) return launch_cheb_tcl(s, dt, st);
         // tensor cores: FP16 split operands (two CTAs per SM) where they fit,
         // else 3xTF32 (one CTA per SM), unless a shape was requested
         if (s.cheb_ept == 16 || (s.cheb_ept == 0 && cheb_tc16_eligible(s.N, s.Ne))) return launch_cheb_tc16(s, dt, st);

@@ -1316,6 +1316,10 @@ iesh_status iesh2_create(iesh2_ctx **out, const iesh2_model *model, int precisio
         d.fx_work_bytes = cheb_fx_work_bytes(N, Ne, max_traj);
         A2(d.fx_work, d.fx_work_bytes)
     }
+    if (ctx->mixed && cheb_tcl_eligible(N, Ne)) {
+        d.fx_work_bytes = cheb_tcl_work_bytes(N, Ne, max_traj);
+        A2(d.fx_work, d.fx_work_bytes)
+    }
     double *mu_d = nullptr;
     float2 *ppdf_d = nullptr;
     if (ctx->nested) A2(mu_d, T * (size_t)(M + 1))
@@ -1333,6 +1337,7 @@ iesh_status iesh2_create(iesh2_ctx **out, const iesh2_model *model, int precisio
     configure_cheb_tc();
     configure_cheb_tc16();
     configure_cheb_fx();
+    configure_cheb_tcl();
     // the slots of the eigen kernel can pass the 48 KiB default (N near 65)
     CU2(raise_smem(k2_eigen<false>, eigen2_smem(N, M, eigen_tpb(N))));
     CU2(raise_smem(k2_eigen<true>, eigen2_smem(N, M, eigen_tpb(N))));
