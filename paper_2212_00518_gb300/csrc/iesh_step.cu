@@ -18,6 +18,7 @@
 #include "iesh_secular.cuh"
 #include "iesh_cheb.cuh"
 #include "iesh_hop.cuh"
+#include "iesh_hop_fx.cuh"
 
 namespace iesh {
 
@@ -1337,7 +1338,10 @@ __global__ void __launch_bounds__(MAXT, MINB) k_hop(DevState s, double dt, doubl
                         G[(int64_t)a * N + m] = gam > 0.0 ? gam : 0.0;
                     }
             }
-        } else {
+        } else if (!hop_fixed(A, dinv, perm, rows, pos_of, isocc, unocc, Ct, N, Ne, scr, [&](int m, int a, double re) {
+                       const double gam = -2.0 * dt * v * re * hop_nac(m, occ_s[a]);
+                       G[(int64_t)a * N + m] = gam > 0.0 ? gam : 0.0;
+                   })) {
             double2 *Y = reinterpret_cast<double2 *>(scr);  // [Ne][N], column m per row
             for (int u0 = 0; u0 < nu; u0 += ngrp) {
                 const int u = u0 + grp;
