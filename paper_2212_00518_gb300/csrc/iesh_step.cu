@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(256) k_build_w(DevState s, double dt, double m
     // j = k + d, d = 1 .. N / 2 (for even N the last d gives each pair twice:
     // half of it); the column sums are read back.  Measured per step, each (j, k)
     // -> each pair: N = 101, 4096 trajectories 3.30 -> 2.09 ms; N = 201, 1024
-    // trajectories 2.69 -> 1.68 ms; N = 21, 64 trajectories 0.067 -> 0.058 ms
+    // trajectories 2.69 -> 1.68 ms; N = 21, 16 trajectories 0.067 -> 0.058 ms
     {
         const int half = N >> 1, pairs = (N & 1) ? half * N : half * N - half;
         int k = threadIdx.x, d = 1;
