@@ -41,10 +41,7 @@ TF32_PER_BF16 = 1.1 / 2.25  # nominal dense TF32 : BF16 tensor rate
 # the named batch size, divided by it: the traffic is per-trajectory streams of C and
 # W, so it scales with the batch.  A shape or kernel not in the table reports null.
 DRAM_BYTES_PER_TRAJ = {
-    # k_cheb, dram__bytes_read.sum + dram__bytes_write.sum of a
-    # 1024-trajectory capture / 1024
-    ("k_cheb", 101, 50): (170.948096e6 + 47.242752e6) / 1024,
-    ("k_cheb", 201, 100): (675.789824e6 + 293.651456e6) / 1024,
+    # no capture of the tensor-core propagators yet
 }
 
 
@@ -277,30 +274,43 @@ def run_ours(args):
         return {k: round(v[0] / tot, 4) for k, v in prof.items() if v[1]}
 
     def fp64_roofline(r, N, Ne):
-        """The FP64 propagator k_cheb against the derived FP64 peak: useful work
-        8 N^2 Ne per trajectory-step (achieved, frac) and executed work K 4 N^2 Ne
-        (executed_*, the FP64 pipe's utilisation)."""
+        """The FP64 propagator: useful work 8 N^2 Ne per trajectory-step
+        (achieved) and the K Chebyshev orders' K 4 N^2 Ne (executed_*).  From
+        N = 28 it is k_cheb_fx, whose product runs as exact FP16 MMAs over
+        fixed-point digits (15 to 28 per useful one), so the peak is the FP16
+        tensor rate; fp64_pipe_frac is the same useful rate against the FP64
+        pipe, which the smaller shapes' k_cheb runs on."""
         n = r["n"]
         pm, pn = r["prof"]["propagate"]
         t = pm / pn / 1e3 if pn else None
         prop_w, step_w = useful_flops(N, Ne)
         ach = prop_w * n / t / 1e12 if t else None
         exe = float(np.sum(r["K"].astype(np.float64))) * 4.0 * N * N * Ne / t / 1e12 if t else None
-        tr = DRAM_BYTES_PER_TRAJ.get(("k_cheb", N, Ne))
+        fx = N >= 28 and N * Ne >= 392  # the library's rule
+        kern = "k_cheb_fx" if fx else "k_cheb"
+        pbf = measured_peaks().get("bf16_tflops")
+        peak = (pbf if pbf else 1900.0) if fx else FP64_NOMINAL_TFLOPS
+        tr = DRAM_BYTES_PER_TRAJ.get((kern, N, Ne))
         step_s = r["ms"] / args.steps / 1e3
-        return {"bound": "alu", "kernel": "k_cheb (Chebyshev exponential integrator, FP64)",
-                "achieved": ach, "peak": FP64_NOMINAL_TFLOPS, "unit": "TFLOP/s",
-                "frac": ach / FP64_NOMINAL_TFLOPS if ach else None,
+        return {"bound": "tensor" if fx else "alu",
+                "kernel": kern + (" (Chebyshev exponential integrator, FP64 in exact fixed point "
+                                  "on the FP16 tensor cores)" if fx else
+                                  " (Chebyshev exponential integrator, FP64)"),
+                "achieved": ach, "peak": peak, "unit": "TFLOP/s",
+                "frac": ach / peak if ach else None,
+                "fp64_pipe_frac": ach / FP64_NOMINAL_TFLOPS if ach else None,
                 "achieved_is": "algorithmic 8 N^2 Ne flops per trajectory-step (unitary "
-                               "application) x trajectories / mean k_cheb launch time",
+                               "application) x trajectories / mean launch time",
                 "executed_achieved": exe,
-                "executed_frac": exe / FP64_NOMINAL_TFLOPS if exe else None,
-                "executed_is": "K 4 N^2 Ne flops actually issued (K Chebyshev orders of a "
+                "executed_frac": exe / peak if exe else None,
+                "executed_is": "K 4 N^2 Ne flops (K Chebyshev orders of a "
                                "real N x N by complex N x Ne product; K over the bulk interval where "
                                "the isolated top level is deflated)",
                 "mean_cheb_terms": float(r["K"].mean()),
-                "peak_source": "derived: 2 DFMA/clk/SM x 152 SMs x 2.07 GHz (no measured FP64 "
-                               "peak in MEASURED_PEAKS.json; a DFMA probe measured 1.20)",
+                "peak_source": (("of measured: MEASURED_PEAKS.json bf16_tflops (FP16 dense = bf16 dense)"
+                                 if pbf else "of fallback: 1.9 PFLOP/s bf16 burst") if fx else
+                                "derived: 2 DFMA/clk/SM x 152 SMs x 2.07 GHz (no measured FP64 "
+                                "peak; a DFMA probe measured 1.20)"),
                 "traffic": tr * n if tr else None,
                 "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum per "
                                   "trajectory of a capture at this shape, times the batch"
@@ -338,6 +348,12 @@ def run_ours(args):
             roof = {"bound": "tensor", "kernel": "k_cheb_tc (tcgen05 kind::tf32, 3xTF32)",
                     "peak": ptf, "peak_source": src,
                     "executed_tensor_tflops": exe * 3 * (128 * Kp * NB) / (N * N * 2 * Ne) if exe else None}
+        elif N > 128 and (Ne >= 16 or (N >= 192 and Ne >= 6)):  # the library's rule
+            pbf = measured_peaks().get("bf16_tflops")
+            roof = {"bound": "tensor", "kernel": "k_cheb_tcl (tcgen05 kind::f16, FP32 as one to three FP16 digits)",
+                    "peak": pbf if pbf else 1900.0,
+                    "peak_source": ("of measured: MEASURED_PEAKS.json bf16_tflops (FP16 dense = bf16 dense)"
+                                    if pbf else "of fallback: 1.9 PFLOP/s bf16 burst")}
         else:
             roof = {"bound": "alu", "kernel": "k_cheb_f32t (register-tiled FP32 SIMT)",
                     "peak": FP32_NOMINAL_TFLOPS,
