@@ -15,10 +15,13 @@
 // column sums of |re| + |im| of U1 and L below 2^b (b <= 4, and below 15) every
 // y and x must stay below 2^l, l = min(60, 62 - b): then no total exceeds 2^62
 // (the first sum may wrap, only the total is used) and the others stay below
-// 2^63.  A row's unit puts its largest entry into [2^(l-4), 2^(l-3)).  The error
-// is about 2^-56.5 of a row's largest entry for b <= 2.  What does not fit --
-// larger entries or sums, a row that grows by more than 8, numbers that are not
-// finite -- goes to the FP64 substitution, from the saved factors.
+// 2^63.  A row's unit puts its largest entry into [2^(l-4), 2^(l-3)), lower by
+// log2 of the largest 1 / |U_kk|, with which the ratios grow.  The error is about
+// 2^-56.5 of a row's largest entry for b <= 2 and pivots near 1.  What does not
+// fit -- larger entries or sums, a row that grows by more than 8 times that,
+// numbers that are not finite -- goes to the FP64 substitution, from the saved
+// factors: of strongly mixed columns (N = 101, Ne = 50) one trajectory in six to
+// one in two, and a trajectory that does so late takes 1.2 times the FP64 time.
 //
 // What bounds it: half of the kernel is now the FP64 factorisation; a product
 // is twelve multiply-adds and some twenty other integer instructions.  Four
@@ -26,7 +29,7 @@
 // factor entries, and 64 rows a pass fill the block.
 // Measured, hop kernel per step: N = 101, Ne = 50, 4096 trajectories 7.70 ->
 // 3.42 ms; N = 201, Ne = 100, 1024 trajectories 13.4 -> 7.6 ms; N = 41, Ne = 20,
-// 1000 trajectories 0.36 -> 0.26 ms; two orbitals, N = 102, 1024 trajectories
+// 1000 trajectories 0.36 -> 0.24 ms; two orbitals, N = 102, 1024 trajectories
 // 2.14 -> 1.06 ms.  With the low products too (sixteen multiply-adds): 3.59 and
 // 8.2 ms for the same errors.
 #pragma once
@@ -101,8 +104,11 @@ __device__ __forceinline__ bool hop_fixed(double2 *A, const double2 *dinv, const
     double2 *saved = reinterpret_cast<double2 *>(scr);                       // [Ne][Ne]
     int4 *Y = reinterpret_cast<int4 *>(saved + (int64_t)Ne * Ne);            // [Ne][nu]
     int4 *F = reinterpret_cast<int4 *>(A);
-    __shared__ int s_big;  // largest column sum; 2^30: outside the range
-    if (tid == 0) s_big = Ne > kHopFxMaxNe ? 1 << 30 : 0;
+    __shared__ int s_big, s_inv;  // largest column sum (2^30: outside the range), key of the largest 1 / U_kk
+    if (tid == 0) {
+        s_big = Ne > kHopFxMaxNe ? 1 << 30 : 0;
+        s_inv = 0;
+    }
     int bad = 0;
     for (int i = tid; i < Ne; i += blockDim.x) {
         off[i] = perm[i] * Ne;
@@ -126,13 +132,16 @@ __device__ __forceinline__ bool hop_fixed(double2 *A, const double2 *dinv, const
         atomicAdd(&(j > k ? sum_u : sum_l)[j], (abs(f.x) >> 10) + (abs(f.z) >> 10) + 2);  // in units of 2^-20
     }
     __syncthreads();
-    int big = bad << 30;
+    int big = bad << 30, inv = 0;
+    for (int i = tid; i < Ne; i += blockDim.x) inv = max(inv, pivot_key(dinv[i]));
+    if (inv) atomicMax(&s_inv, inv);
     for (int i = tid; i < Ne; i += blockDim.x) big = max(big, max(sum_u[i], sum_l[i]));
     if (big) atomicMax(&s_big, big);
     __syncthreads();
     big = s_big;
     bad = big >= 15 << 20;
     const int l = min(60, 62 - (32 - __clz(big >> 20)));
+    const int room = 4 + max(0, min(12, (s_inv >> 20) - 1023));
     const int sub = tid & 3, grp = tid >> 2, ngrp = blockDim.x >> 2;
     const unsigned quad = 0xFu << (lane & ~3);
     if (!bad)
@@ -153,7 +162,7 @@ __device__ __forceinline__ bool hop_fixed(double2 *A, const double2 *dinv, const
                 bad = 1;
                 e = 0;
             }
-            const double up = __hiloint2double((1023 + l - 4 - e) << 20, 0), down = __hiloint2double((1023 - l + 4 + e) << 20, 0);
+            const double up = __hiloint2double((1023 + l - room - e) << 20, 0), down = __hiloint2double((1023 - l + room + e) << 20, 0);
             if (live && !bad)
                 for (int i = sub; i < Ne; i += 4) {
                     const double2 c = Ct[(int64_t)i * N + m];
