@@ -166,12 +166,14 @@ __device__ __forceinline__ dfl nested_gap(const Poles<R> &P, int o, int k, dfl t
 // z_k q0 / (lam - eps_k).  Each root is found in the shifted variable
 // tau = lam - eps_o relative to its nearer pole o, so lam - eps_k =
 // (eps_o - eps_k) + tau keeps full relative accuracy.
-// gp = gp_rest + the origin's share; s3 = sum_k z_k^2 / (lam - eps_k)^3
-// (FP32, where the mode forms it), so g'' = -2 s3; sabs = the scale of g's
-// rounding error.
+// gp = gp_rest + the origin's share; rt = 1 / tau; s3 = sum over k != o of
+// z_k^2 / (lam - eps_k)^3 (FP32, where the mode forms it), so g'' = -2 (s3 +
+// (gp - gp_rest) rt): the origin's share, of order gap^3 / z^4, leaves FP32's
+// range once z^2 is below about 10^-21 (a coupling that decays to 10^-8 of its
+// value) and is formed in R.  sabs = the scale of g's rounding error.
 template <class R>
 struct Sec {
-    R g, gp, gp_rest, qo, sabs;
+    R g, gp, gp_rest, qo, rt, sabs;
     float s3;
 };
 
@@ -247,8 +249,9 @@ __device__ __forceinline__ Sec<R> sec_eval(const Poles<R> &P, int o, R tau, R eo
         float f1 = 0.f, f2 = 0.f, fa = 0.f;
 #pragma unroll 4
         for (int k = 0; k < M; ++k) {
-            const float r = pole_recip<float>((po - P.hdf[k].x) + tf);
-            const float v = k != o ? P.z2df[k].x * r : 0.f, w = v * r;
+            // (the origin's distance may be below FP32's range)
+            const float r = k != o ? pole_recip<float>((po - P.hdf[k].x) + tf) : 0.f;
+            const float v = P.z2df[k].x * r, w = v * r;
             f1 += v;
             f2 += w;
             fa += fabsf(v);
@@ -285,8 +288,9 @@ __device__ __forceinline__ Sec<R> sec_eval(const Poles<R> &P, int o, R tau, R eo
     e.gp_rest = R(1) + s2;
     e.gp = e.gp_rest + wo;
     e.qo = qo;
+    e.rt = rt;
     e.sabs = sa;
-    e.s3 = fmaf((float)wo, (float)rt, s3);
+    e.s3 = s3;
     return e;
 }
 
@@ -336,17 +340,19 @@ __device__ __forceinline__ R sec_delta(int kind, const Sec<R> &e, R s, R tau, R 
 }
 
 // A correction this small against the distance to the nearer end of the gap
-// ends the iteration: tau takes it, and gp its first-order change -2 s3 delta
-// (what is left out is of second order, below the mode's rounding).  FP32:
-// 2^-13; double-float sums: 2^-23; the last FP64 evaluation of a staged
-// solve: 2^-31.
+// ends the iteration: tau takes it, and gp its first-order change g'' delta
+// (what is left out is of second order, below the mode's rounding; the change
+// is at most 2 limit gp, so a larger one is an overflow).  FP32: 2^-13;
+// double-float sums: 2^-23; the last FP64 evaluation of a staged solve: 2^-31.
 template <class R>
 __device__ __forceinline__ bool sec_accept(int kind, R D, R limit, R delta, R &tau, Sec<R> &e)
 {
     const R tp = kind == 0 ? tau - D : tau + D;
     const R dist = kind <= 1 ? fmin(fabs(tau), fabs(tp)) : fabs(tau);
     if (!(fabs(delta) <= limit * dist)) return false;
-    e.gp += (R)(-2.0f * e.s3 * (float)delta);
+    const R change = R(-2) * ((e.gp - e.gp_rest) * (delta * e.rt) + (R)(e.s3 * (float)delta));
+    if (!(fabs(change) <= R(1e-3) * e.gp)) return false;
+    e.gp += change;
     tau += delta;
     return true;
 }
@@ -438,6 +444,7 @@ __device__ void secular_root(int r, const Poles<R> &P, R h, R Z2, bool warm, R g
                 e.gp_rest += (e.gp - e.gp_rest) - qr * rd;
                 e.sabs += fabs(qL) - fabs(qr);
                 e.qo = qr;
+                e.rt = rd;
             }
             // coarser sums may misjudge a root near the middle: the later
             // stages get the whole gap
