@@ -6,7 +6,11 @@
 // FMAs and the quads' reductions) were 77% of the kernel.  A complex product
 // of 57-bit integers is twelve 32 x 32 -> 64 multiply-adds on the integer pipe.
 //
-// With P S = L U and D = diag U: x = c U1^{-1} D^{-1} L^{-1}, U1 = D^{-1} U.
+// With P S = L U, column j of S and of the rows c scaled by 2^p_j, p_j the
+// exponent of 1 / U_jj (the ratios do not change), U' = U diag(2^p) and D' =
+// diag U', 1 / D' with entries in [1, 2.9): x = c diag(2^p) U1^{-1} D'^{-1}
+// L^{-1}, U1 = D'^{-1} U'.  So no pivot multiplies the rounding of a row, and a
+// scaled electron gives the same bits.
 // U1 and L are held as a = a1 2^26 + a0, |a0| <= 2^25, in the unit 2^-56 (their
 // entries must be below 1.75), a row as y = y1 2^30 + y0, |y0| <= 2^29.  A sum of
 // products in y's unit is
@@ -15,13 +19,14 @@
 // column sums of |re| + |im| of U1 and L below 2^b (b <= 4, and below 15) every
 // y and x must stay below 2^l, l = min(60, 62 - b): then no total exceeds 2^62
 // (the first sum may wrap, only the total is used) and the others stay below
-// 2^63.  A row's unit puts its largest entry into [2^(l-4), 2^(l-3)), lower by
-// log2 of the largest 1 / |U_kk|, with which the ratios grow.  The error is about
-// 2^-56.5 of a row's largest entry for b <= 2 and pivots near 1.  What does not
-// fit -- larger entries or sums, a row that grows by more than 8 times that,
+// 2^63.  A row's unit puts its largest scaled entry into [2^(l-4), 2^(l-3)); a row
+// that grows past 2^l is formed again in a unit 2^3 larger, up to three times.
+// The error is about 2^-56.5 of a row's largest entry, on the way or in the
+// result, for b <= 2: a slot whose ratios are far below the row's others keeps
+// that absolute error (10^-6 of them: 10^-10 of the slot's own, where FP64 had
+// 10^-15).  What does not fit -- larger entries or sums, rows that grow further,
 // numbers that are not finite -- goes to the FP64 substitution, from the saved
-// factors: of strongly mixed columns (N = 101, Ne = 50) one trajectory in six to
-// one in two, and a trajectory that does so late takes 1.2 times the FP64 time.
+// factors; entries and sums are known before the first row.
 //
 // What bounds it: half of the kernel is now the FP64 factorisation; a product
 // is twelve multiply-adds and some twenty other integer instructions.  Four
@@ -94,21 +99,20 @@ __device__ __forceinline__ int fx_out(long long n, int l) { return ((int)(n >> l
 // Substitutes all unoccupied rows; emit(m, a, Re (C_m S^{-1})_a) for each
 // entry.  A, dinv, perm: the factors as k_hop leaves them; off, sum_u and
 // sum_l [Ne]: shared, free; scr: 2 Ne N doubles.  All threads of the CTA
-// call it after a barrier.  False: A is unchanged and the entries that were
-// emitted are to be formed again.
+// call it after a barrier.  False: A and dinv are unchanged and the entries
+// that were emitted are to be formed again.
 template <class Emit>
-__device__ __forceinline__ bool hop_fixed(double2 *A, const double2 *dinv, const int *perm, int *off, int *sum_u, int *sum_l,
+__device__ __forceinline__ bool hop_fixed(double2 *A, double2 *dinv, const int *perm, int *off, int *sum_u, int *sum_l,
                                           const int *unocc, const double2 *Ct, int N, int Ne, double *scr, Emit emit)
 {
     const int nu = N - Ne, tid = threadIdx.x, lane = tid & 31;
     double2 *saved = reinterpret_cast<double2 *>(scr);                       // [Ne][Ne]
     int4 *Y = reinterpret_cast<int4 *>(saved + (int64_t)Ne * Ne);            // [Ne][nu]
     int4 *F = reinterpret_cast<int4 *>(A);
-    __shared__ int s_big, s_inv;  // largest column sum (2^30: outside the range), key of the largest 1 / U_kk
-    if (tid == 0) {
-        s_big = Ne > kHopFxMaxNe ? 1 << 30 : 0;
-        s_inv = 0;
-    }
+    static_assert(kMaxHopElectrons <= kHopFxMaxNe, "28 products per lane at most");
+    __shared__ int s_big;  // largest column sum (2^30: outside the range)
+    if (tid == 0) s_big = 0;
+    auto exponent = [&](int j) { return (pivot_key(dinv[j]) >> 20) - 1023; };  // p_j
     int bad = 0;
     for (int i = tid; i < Ne; i += blockDim.x) {
         off[i] = perm[i] * Ne;
@@ -121,27 +125,39 @@ __device__ __forceinline__ bool hop_fixed(double2 *A, const double2 *dinv, const
         double2 v = A[at];
         saved[at] = v;
         if (j == k) continue;
-        if (j > k) v = cmul(v, dinv[k]);
-        if (pivot_key(v) >= 0x3ffc0000) {  // 1.75 or more, or not finite
+        int d = 0;  // U1 = U_kj / U_kk 2^(p_j - p_k)
+        if (j > k) {
+            v = cmul(v, dinv[k]);
+            d = max(-800, min(800, exponent(j) - exponent(k)));
+        }
+        if (pivot_key(v) >= 0x3ffc0000 - d * (1 << 20)) {  // 1.75 or more, or not finite
             bad = 1;
             continue;
         }
-        const double sc = 72057594037927936.0;  // 2^56
+        const double sc = __hiloint2double((1023 + 56 + d) << 20, 0);
         const int4 f = fx_pack<26>(__double2ll_rn(v.x * sc), __double2ll_rn(v.y * sc));
         F[at] = f;
         atomicAdd(&(j > k ? sum_u : sum_l)[j], (abs(f.x) >> 10) + (abs(f.z) >> 10) + 2);  // in units of 2^-20
     }
     __syncthreads();
-    int big = bad << 30, inv = 0;
-    for (int i = tid; i < Ne; i += blockDim.x) inv = max(inv, pivot_key(dinv[i]));
-    if (inv) atomicMax(&s_inv, inv);
-    for (int i = tid; i < Ne; i += blockDim.x) big = max(big, max(sum_u[i], sum_l[i]));
+    int big = bad << 30;
+    for (int i = tid; i < Ne; i += blockDim.x) {
+        big = max(big, max(sum_u[i], sum_l[i]));
+        int p = exponent(i);
+        if (p > 400 || p < -400) {
+            big = 1 << 30;
+            p = 0;
+        }
+        sum_u[i] = p;
+        const double sc = __hiloint2double((1023 - p) << 20, 0);
+        dinv[i] = make_double2(dinv[i].x * sc, dinv[i].y * sc);  // 1 / U'_ii
+    }
     if (big) atomicMax(&s_big, big);
     __syncthreads();
     big = s_big;
     bad = big >= 15 << 20;
+    const int *unit = sum_u;  // p_j
     const int l = min(60, 62 - (32 - __clz(big >> 20)));
-    const int room = 4 + max(0, min(12, (s_inv >> 20) - 1023));
     const int sub = tid & 3, grp = tid >> 2, ngrp = blockDim.x >> 2;
     const unsigned quad = 0xFu << (lane & ~3);
     if (!bad)
@@ -150,22 +166,26 @@ __device__ __forceinline__ bool hop_fixed(double2 *A, const double2 *dinv, const
             const bool live = u < nu;
             const int m = live ? unocc[u] : 0;
             int4 *y = Y + (live ? u : 0);
-            // the row's unit, and the row in it
-            int mx = 0;
+            // the exponent of the row's largest scaled entry
+            int e = -4096;
             if (live)
-                for (int i = sub; i < Ne; i += 4) mx = max(mx, pivot_key(Ct[(int64_t)i * N + m]));
-            mx = max(mx, __shfl_xor_sync(quad, mx, 1));
-            mx = max(mx, __shfl_xor_sync(quad, mx, 2));
-            int e = (mx >> 20) - 1023;
-            if (mx == 0) e = 0;
-            if (e > 900 || e < -900) {
+                for (int i = sub; i < Ne; i += 4) {
+                    const int key = pivot_key(Ct[(int64_t)i * N + m]);
+                    if (key) e = max(e, key >= 0x7ff00000 ? 4096 : (key >> 20) - 1023 + unit[i]);
+                }
+            e = max(e, __shfl_xor_sync(quad, e, 1));
+            e = max(e, __shfl_xor_sync(quad, e, 2));
+            if (e == -4096) e = 0;
+            int room = 4, out = 0;  // of this row
+            if (e > 500 || e < -500) {
                 bad = 1;
                 e = 0;
             }
-            const double up = __hiloint2double((1023 + l - room - e) << 20, 0), down = __hiloint2double((1023 - l + room + e) << 20, 0);
+          again:
             if (live && !bad)
                 for (int i = sub; i < Ne; i += 4) {
                     const double2 c = Ct[(int64_t)i * N + m];
+                    const double up = __hiloint2double((1023 + l - room - e + unit[i]) << 20, 0);
                     *reinterpret_cast<longlong2 *>(y + i * nu) = make_longlong2(__double2ll_rn(c.x * up), __double2ll_rn(c.y * up));
                 }
             __syncwarp(quad);
@@ -181,18 +201,18 @@ __device__ __forceinline__ bool hop_fixed(double2 *A, const double2 *dinv, const
                     const longlong2 c = *reinterpret_cast<const longlong2 *>(y + jc * nu);
                     re = c.x - re;
                     im = c.y - im;
-                    bad |= fx_out(re, l) | fx_out(im, l);
+                    out |= fx_out(re, l) | fx_out(im, l);
                     y[jc * nu] = fx_pack<30>(re, im);
                 }
                 __syncwarp(quad);
             }
-            // y D^{-1}
+            // y D'^{-1}
             if (live)
                 for (int i = sub; i < Ne; i += 4) {
                     const int4 v = y[i * nu];
                     const double2 r = cmul(make_double2((double)fx_join(v.x, v.y), (double)fx_join(v.z, v.w)), dinv[i]);
                     if (pivot_key(r) >= (1023 + l) << 20) {
-                        bad = 1;
+                        out = 1;
                         y[i * nu] = make_int4(0, 0, 0, 0);
                     } else {
                         y[i * nu] = fx_pack<30>(__double2ll_rn(r.x), __double2ll_rn(r.y));
@@ -211,11 +231,21 @@ __device__ __forceinline__ bool hop_fixed(double2 *A, const double2 *dinv, const
                     const int4 v = y[jc * nu];
                     re = fx_join(v.x, v.y) - re;
                     im = fx_join(v.z, v.w) - im;
-                    bad |= fx_out(re, l) | fx_out(im, l);
+                    out |= fx_out(re, l) | fx_out(im, l);
                     y[jc * nu] = fx_pack<30>(re, im);
                 }
                 __syncwarp(quad);
             }
+            // (a row that has been given up is of no further use)
+            if (__any_sync(quad, out) && !bad) {
+                if (room < 13) {
+                    room += 3;
+                    out = 0;
+                    goto again;
+                }
+                bad = 1;
+            }
+            const double down = __hiloint2double((1023 - l + room + e) << 20, 0);
             if (live)
                 for (int i = sub; i < Ne; i += 4) {
                     const int4 v = y[i * nu];
@@ -223,8 +253,13 @@ __device__ __forceinline__ bool hop_fixed(double2 *A, const double2 *dinv, const
                 }
         }
     bad = __syncthreads_or(bad);
-    if (bad)
+    if (bad) {
         for (int idx = tid; idx < Ne * Ne; idx += blockDim.x) A[idx] = saved[idx];
+        for (int i = tid; i < Ne; i += blockDim.x) {  // (exact)
+            const double sc = __hiloint2double((1023 + unit[i]) << 20, 0);
+            dinv[i] = make_double2(dinv[i].x * sc, dinv[i].y * sc);
+        }
+    }
     __syncthreads();
     return !bad;
 }
