@@ -77,8 +77,9 @@ __device__ inline int cheb_terms(double rho, double tol)
 
 // Bound on the amplification, by the series over [c - rho, c + rho], of a
 // component along an eigenvector whose eigenvalue mu lies outside it:
-// |J_0| + 2 sum_{k=1..K} |J_k(rho)| |T_k(mu_x)|, mu_x = (mu - c) / rho.
-__device__ inline double cheb_amplification(const double *cb, double mu)
+// |J_0| + 2 sum_{k=1..K} |J_k(rho)| |T_k(mu_x)|, mu_x = (mu - c) / rho > 1.
+// tmax: the largest |T_k(mu_x)|, which is T_K's.
+__device__ inline double cheb_amplification(const double *cb, double mu, double &tmax)
 {
     const double c = cb[0], rho = cb[1];
     const int K = (int)cb[2];
@@ -91,6 +92,7 @@ __device__ inline double cheb_amplification(const double *cb, double mu)
         tm = tk;
         tk = tn;
     }
+    tmax = fabs(tm);
     return A;
 }
 

@@ -312,14 +312,6 @@ __global__ void __launch_bounds__(kTlThreads, 2)
             }
             if (defl && tid < ne) s_a[tid] = make_float2(dq[2 * N + e0 + tid], dq[2 * N + Ne + e0 + tid]);
             __syncthreads();  // (s_max is zero)
-            if (defl)  // c - a u
-#pragma unroll
-                for (int q = 0; q < kTlMaxCols / 2; ++q)
-                    if (rowok && q < ne) {
-                        const float2 a = s_a[q];
-                        tk[2 * q] -= fmaf(a.x, ur, -(a.y * ui));
-                        tk[2 * q + 1] -= fmaf(a.x, ui, a.y * ur);
-                    }
             if (wact) {
                 int mm[kTlMaxEl];
 #pragma unroll
@@ -331,6 +323,14 @@ __global__ void __launch_bounds__(kTlThreads, 2)
                 for (int q = 0; q < kTlMaxEl; ++q) mine = lane == q ? mm[q] : mine;
                 if (lane < kTlMaxEl) atomicMax(&s_max[lane], mine);
             }
+            if (defl)  // c - a u (the scales are those of c: the share along u grows)
+#pragma unroll
+                for (int q = 0; q < kTlMaxCols / 2; ++q)
+                    if (rowok && q < ne) {
+                        const float2 a = s_a[q];
+                        tk[2 * q] -= fmaf(a.x, ur, -(a.y * ui));
+                        tk[2 * q + 1] -= fmaf(a.x, ui, a.y * ur);
+                    }
             __syncthreads();
             if (wact) {
                 const float J0 = s_cj[0];

@@ -230,19 +230,33 @@ __global__ void k_force(DevState s)
 constexpr int kDeflIter = 48;
 constexpr int kDeflGain = 2;
 constexpr double kDeflAmp64 = 1e3, kDeflAmp32 = 16.0;
+// What is left of a column along u -- the rounding of c - a u (2^-52 of the
+// column, FP32 2^-24) and u's own error, at most its residual over its distance
+// to the bulk -- grows with T_k(mu_x), up to 10^3 / tol.  That is harmless where T_k
+// has a floating point's range; the tensor-core kernels hold it in fixed point
+// (FP64: entries below 2, columns normalised to 1 to 2) and in FP16 digits
+// (mixed, N > 128: norms scaled to at most 2^14.5, digits end at 2^16), so they
+// also ask that the share stays below kDeflShare of the column (each order's
+// rounding adds about as much).  On the double well T_k(mu_x) is 4e10 at dt = 1
+// and 2e14 at dt = 3 (tol 1e-15), 6e5 at dt = 1 and 3e6 at 1.5 (1e-7).
+constexpr double kDeflShare = 0.25;
 
 // Thread 0 has set up the series over the bulk interval; it keeps the
 // deflation if the series amplifies the u direction by at most amp, else it
 // sets the full interval up.  Returns the block-uniform decision.
+// unit: rounding of the deflated columns; res / den: u's squared residual.
 // rtop: the top row's Gershgorin radius.  The FP64 propagator's fixed-point
 // ranges also ask that the top row's couplings and diagonal stay within 8 and
 // 10^6 bulk half-widths (rows inside the interval have at most 1).
 __device__ inline bool defl_keep(const DevState &s, int64_t t, bool deflate, double mu, double lo, double hi,
-                                 double tol, double amp, double rtop, double *df, int *flag)
+                                 double tol, double amp, double unit, double res, double den, double rtop, double *df,
+                                 int *flag)
 {
     if (threadIdx.x == 0) {
         const double *cb = s.cheb + t * kChebStride;
-        bool k = deflate && cheb_amplification(cb, mu) <= amp && rtop <= 8.0 * cb[1] && mu - cb[0] <= 1e6 * cb[1];
+        double tmax = 0.0;
+        bool k = deflate && cheb_amplification(cb, mu, tmax) <= amp && rtop <= 8.0 * cb[1] && mu - cb[0] <= 1e6 * cb[1];
+        if (k && s.fx_work) k = tmax * (unit + sqrt(res / den) / (mu - cb[0] - cb[1])) <= kDeflShare;
         if (deflate && !k) cheb_setup(s, t, lo, hi, tol);
         *flag = k;
         if (df) {
@@ -314,7 +328,7 @@ __global__ void __launch_bounds__(256) k_build_w(DevState s, double dt, double m
     hi = block_max(hi, red);
     double *df = s.defl ? s.defl + t * defl_stride(N, s.Ne) : nullptr;
     bool deflate = false;
-    double hb = hi, mu = 0.0;
+    double hb = hi, mu = 0.0, res_u = 0.0, den_u = 1.0;
     if (df && N >= 3 && N <= (int)blockDim.x) {
         const int top = N - 1;  // eigenvalues ascending at both ends: L is ascending
         double b = -__longlong_as_double(0x7ff0000000000000ll);
@@ -335,6 +349,7 @@ __global__ void __launch_bounds__(256) k_build_w(DevState s, double dt, double m
                 ui[j] = 0.0;
             }
             __syncthreads();
+            bool last = false;
             for (int it = 0; it < kDeflIter; ++it) {
                 double hr = 0.0, hv = 0.0;
                 if (rj) {
@@ -360,9 +375,15 @@ __global__ void __launch_bounds__(256) k_build_w(DevState s, double dt, double m
                 const double er = rj ? fma(-m, ur[j], hr) : 0.0, ei = rj ? fma(-m, ui[j], hv) : 0.0;
                 const double res = block_sum(fma(er, er, ei * ei), red);
                 const double gap = m - sigma;
-                if (res <= 1e-28 * gap * gap * den) {  // uniform: every thread holds the same sums
+                // (the fixed-point propagator's test of u, in defl_keep, may want
+                // what one more correction gives)
+                const bool more = s.fx_work && !last && res > 1e-31 * gap * gap * den;
+                if (res <= 1e-28 * gap * gap * den) last = true;
+                if (last && !more) {  // uniform: every thread holds the same sums
                     deflate = gap > 0.0;
                     mu = m;
+                    res_u = res;
+                    den_u = den;
                     if (rj) {
                         const double inv = 1.0 / sqrt(den);
                         ur[j] *= inv;
@@ -382,7 +403,9 @@ __global__ void __launch_bounds__(256) k_build_w(DevState s, double dt, double m
     }
     if (threadIdx.x == 0) cheb_setup(s, t, lo, hb, tol);
     __shared__ int keep;
-    if (!defl_keep(s, t, deflate, mu, lo, hi, tol, kDeflAmp64, deflate ? Lk_s[N - 1] - hb_s[N - 1] : 0.0, df, &keep)) return;
+    if (!defl_keep(s, t, deflate, mu, lo, hi, tol, kDeflAmp64, 0x1p-52, res_u, den_u,
+                   deflate ? Lk_s[N - 1] - hb_s[N - 1] : 0.0, df, &keep))
+        return;
     const int Ne = s.Ne;
     double *q = df + kDeflHead;
     for (int j = threadIdx.x; j < N; j += blockDim.x) {
@@ -571,7 +594,7 @@ __global__ void __launch_bounds__(256, 5) k_build_w_f32(DevState s, double dt, d
     if (threadIdx.x == 0) cheb_setup(s, t, lo, hb, tol);
     if (!dfl) return;
     __shared__ int keep;
-    if (!defl_keep(s, t, deflate, mu, lo, hi, tol, kDeflAmp32, 0.0, df, &keep)) return;
+    if (!defl_keep(s, t, deflate, mu, lo, hi, tol, kDeflAmp32, 0x1p-24, 0.0, 1.0, 0.0, df, &keep)) return;
     const int Ne = s.Ne;
     float *q = reinterpret_cast<float *>(df + kDeflHead);  // packed floats
     for (int j = threadIdx.x; j < N; j += blockDim.x) {
