@@ -350,7 +350,7 @@ def run_ours(args):
                     "executed_tensor_tflops": exe * 3 * (128 * Kp * NB) / (N * N * 2 * Ne) if exe else None}
         elif N > 128 and (Ne >= 16 or (N >= 192 and Ne >= 6)):  # the library's rule
             pbf = measured_peaks().get("bf16_tflops")
-            roof = {"bound": "tensor", "kernel": "k_cheb_tcl (tcgen05 kind::f16, FP32 as one to three FP16 digits)",
+            roof = {"bound": "tensor", "kernel": "k_cheb_tcl (tcgen05 kind::f16, FP32 as two or three FP16 digits)",
                     "peak": pbf if pbf else 1900.0,
                     "peak_source": ("of measured: MEASURED_PEAKS.json bf16_tflops (FP16 dense = bf16 dense)"
                                     if pbf else "of fallback: 1.9 PFLOP/s bf16 burst")}
@@ -372,7 +372,8 @@ def run_ours(args):
 
     MIXED_DTYPE = ("f32 coefficients, coupling generator, propagation (tensor cores for N <= 128: "
                    "FP16 hi + lo split operands, about 22 bits each, FP32 accumulation, where two CTAs "
-                   "fit an SM, else 3xTF32; FP32 SIMT above), overlap LU or Gauss-Jordan ratios; "
+                   "fit an SM, else 3xTF32; above, two or three FP16 digits of FP32 operands, at least "
+                   "24 bits, or FP32 SIMT for few electrons), overlap LU or Gauss-Jordan ratios; "
                    "double-float secular sums; f64 eigen iteration, forces, hop selection and rescale")
 
     # ---------------------------------------------- headline: M = args.M

@@ -7,30 +7,32 @@
 // as FP16 MMAs with FP32 accumulation.  Both operands are FP32 numbers split
 // into FP16 digits of 11 bits (x = x_0 + x_1 + x_2, each the FP16 rounding of
 // what is left), scaled so that the largest entry of W' = (2 / rho) W and
-// every electron column's norm lie near the top of the FP16 range.  With |W'|
-// < 2^(e+1) the product of digits i and j is about 2^(e - 11 (i + j)) of T:
-// the pairs i + j <= s are formed, s = floor((28 + e) / 11) at most 2, so
-// that what is left out stays below 2^-28 of a column's norm -- six products
-// for couplings of order 1, three below 2^-6, one below 2^-17 (the bath
-// levels of the double well couple at 10^-6 per step).  The SIMT kernel
-// rounds T_k to 2^-25 of its entries.
+// every electron column's norm lie near the top of the FP16 range.  Two digits
+// of both operands (three products) hold 24 bits: the amplitude of an empty
+// orbital, which W' T makes, then has FP32's accuracy however weak the
+// couplings are (one step from unit columns, N = 201: hop probabilities within
+// 3e-7 of the largest, as FP32 products give; one digit gave 5e-4).  With |W'| <
+// 2^(e+1) the product of digits i and j is about 2^(e - 11 (i + j)) of T, and
+// what is left out stays below 2^-28 of a column's norm: three digits (six
+// products) from |W'| = 2^-6 up.  The SIMT kernel rounds T_k to 2^-25 of its
+// entries.
 //
 // Two persistent CTAs of 256 threads (one per row) per SM take (trajectory,
 // electron range) items in blocks of up to 16 electrons (32 real columns), in
 // the layouts of k_cheb_fx (iesh_cheb_fx.cu).  T_k and T_{k-1} are in registers
 // (32 values each per thread), the product and the Chebyshev sum in tensor
 // memory, T's digits in shared memory.  W' is cut into digits once per item:
-// with one digit (and at most 14 K steps) straight into shared memory, where it
-// stays for all blocks and orders; otherwise into the CTA's slot of a workspace
+// where they fit (N up to about 135) straight into shared memory, where they
+// stay for all blocks and orders; otherwise into the CTA's slot of a workspace
 // that stays in L2, streamed back by bulk copies through a ring of two or three
 // slots of several K steps.
 //
-// What bounds it: the chain of an order -- barrier, MMAs (26 of 128 x 32 x 16
+// What bounds it: the chain of an order -- barrier, MMAs (78 of 128 x 32 x 16
 // at N = 201, 41 cycles each), commit, wait, update of the registers and
-// digits -- of two CTAs that fill each other's waits; neither the tensor cores
-// (10%), the FP32 pipe (20%) nor memory (7%) is busy.  Measured at N = 201,
+// digits -- of two CTAs that fill each other's waits.  Measured at N = 201,
 // Ne = 100, 8192 trajectories, 5 orders: 17.0 ms per step for the SIMT kernel
-// (50% of the FP32 peak) -> 7.4 ms.  One CTA of 512 threads per SM: 17.6 ms
+// (50% of the FP32 peak) -> 8.4 ms (7.35 with one digit, 11.8 with three, which
+// is not more accurate).  One CTA of 512 threads per SM took 17.6 ms
 // with a commit per K step and row tile, 10.9 ms with several K steps per slot.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -97,7 +99,7 @@ __device__ __forceinline__ bool tl_order(TlMma &m, uint32_t &fpar, bool ring)
         }
         uint64_t ak = m.ad0 + sl * (m.kps * m.kstep);
         const uint32_t k1 = min(m.ks, k0 + m.kps);
-#pragma unroll(NSL == 1 ? 4 : 1)
+#pragma unroll 1
         for (uint32_t k = k0; k < k1; ++k, ak += m.kstep, bd += 16)
 #pragma unroll
             for (int tl = 0; tl < 2; ++tl)
@@ -225,7 +227,7 @@ __global__ void __launch_bounds__(kTlThreads, 2)
         int e = (int)((__float_as_int(wmax) >> 23) & 0xff) - 127;
         if (e > 100) e = 0;
         if (e < -60) e = -60;
-        const int nsl = min(kTlS, max(1, 1 + (28 + e >= 0 ? (28 + e) / 11 : 0)));
+        const int nsl = e >= -6 ? kTlS : 2;
         const float ws_scale = w2 * __int_as_float((127 + 13 - e) << 23);  // digits of 2^(13 - e) W'
         const float dscale = __int_as_float((127 + e - 27) << 23);         // D of 2^14 T from the accumulator: 2^(e - 13)
         const float d14 = dscale * 16384.0f;
@@ -358,11 +360,7 @@ __global__ void __launch_bounds__(kTlThreads, 2)
                 tc::fence_after_sync();
                 if (warp == 0) {
                     if (tc::elect_one()) {
-                        switch (nsl) {
-                        case 1: ok = tl_order<1>(m, fpar, !resident); break;
-                        case 2: ok = tl_order<2>(m, fpar, !resident); break;
-                        default: ok = tl_order<3>(m, fpar, !resident); break;
-                        }
+                        ok = nsl == 2 ? tl_order<2>(m, fpar, !resident) : tl_order<3>(m, fpar, !resident);
                         tc::commit(&done);
                     }
                     __syncwarp();
