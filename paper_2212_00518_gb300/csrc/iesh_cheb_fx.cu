@@ -14,11 +14,11 @@
 //   W' = 2^e sum_i W_i 2^{-8-8i},  T = sum_j T_j 2^{-8-8j},  i, j = 0..6,
 // integers |W_0|, |T_0| <= 512 and |W_i|, |T_j| <= 128, each stored as an
 // FP16 value.  The products of one weight, i + j = g, share one FP32
-// accumulator in tensor memory (groups g = 0..G, G <= 6, 28 products at
-// most); an accumulator stays an exact integer (Cauchy-Schwarz, with the
-// columns' unit norm: below 2^24 for N <= 128, and beyond that unless every
-// digit of a row and a column aligns in sign).  The update reads the group
-// sums, adds them as 64-bit integers and forms
+// accumulator in tensor memory (groups g = 0..G, G = 5 or 6, 28 products at
+// most); an accumulator is an exact integer as long as it stays below 2^24
+// (digits of random sign give 2^18 at N = 128; only digits aligned in sign along
+// a whole row and column pass it, and then round in the last of 24 bits).  The
+// update reads the group sums, adds them as 64-bit integers and forms
 //   T_{k+1} = 2 (L - c) / rho T_k - i W' T_k - T_{k-1}
 // in integer arithmetic; the Chebyshev sum is a 64-bit integer as well.
 //
@@ -26,7 +26,13 @@
 // against the FP64 kernel's rounding of 2^-54 .. 2^-57 of typical entries.
 // The terms left out (i + j > G) amount to about 2^{17.5 - 16 - 8 (G+1) + e}:
 // G is the smallest value that brings this to 2^-56, at most 6 (2^-54.5 for
-// |W'| of order 1).  Weak couplings (small e) need fewer products.
+// |W'| of order 1).  Couplings so weak that an entry which starts from zero
+// stays small give every entry a unit of its own, up to 2^16 finer (a byte per
+// entry, from its size and a bound of its growth), and G = 5, 2^-46.5 of max |W'|:
+// the amplitude of an empty orbital after a step from unit columns, of the size
+// of W', then carries 2e-14 of the largest of them and 10^-12 of its own (N = 101,
+// dt = 1; one unit per column: 2e-11 and 2e-9; FP64 arithmetic: 2e-16).  Couplings
+// below 2^-75 of the interval vanish.
 //
 // Layout.  One persistent CTA of 512 threads per SM takes (trajectory, range
 // of electrons) items, in blocks of up to 64 real columns for one 128-row
@@ -41,12 +47,12 @@
 // T_k and T_{k-1} are in registers (up to 16 values each per thread).
 //
 // Measured (ms per step, against the SIMT kernel): N = 101, Ne = 50, 4096
-// trajectories 6.5 against 65.7; N = 201, Ne = 100, 1024 trajectories 9.6
-// against 127; N = 41, Ne = 20, 1000 trajectories, 20 orders 1.17 against
-// 2.76.  Per order and 64 columns at N = 101 (5 digits) the MMAs take 8.5k
-// cycles and the update 10k; neither overlaps the other (tensor memory holds
-// one block), and the update's 64-bit integer arithmetic, about 100
-// instructions per entry, is latency-bound at 4 warps per scheduler.
+// trajectories 7.5 against 65.7; N = 201, Ne = 100, 1024 trajectories 12.6
+// against 127; N = 41, Ne = 20, 1000 trajectories, 20 orders 1.23 against
+// 2.76.  (One unit per column and G = 4 for weak couplings: 6.4, 9.5 and 1.17.)
+// MMAs and update do not overlap (tensor memory holds one block); the update's
+// 64-bit integer arithmetic, about 100 instructions per entry, is
+// latency-bound at 4 warps per scheduler.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -64,10 +70,13 @@ constexpr int kFxWarps = kFxThreads / 32;
 constexpr int kFxS = 7;               // digits of each operand
 constexpr int kFxMaxCols = 16;        // real columns per thread
 constexpr int kFxMaxEl = 32;          // electrons per block
+constexpr int kFxMaxShift = 16;       // of an entry's unit below 2^-60
 constexpr int kFxWaitLimit = 1 << 22;
 constexpr int kFxMaxStages = 16;
 constexpr size_t kFxMaxSmem = 220 * 1024;
-constexpr int kFxSlack = 4096;        // an MMA reads 16 row groups from a digit's start
+// at the end of the shared memory: the threads' shifts, 8 bytes each; an MMA
+// reads 16 row groups from a digit's start, up to there (rows that are not used)
+constexpr int kFxSlack = kFxThreads * 8;
 
 // Sizes: rg 8-row groups of W, row tiles of 128 rows, ks K steps of 16.
 struct FxShape {
@@ -115,6 +124,16 @@ __device__ __forceinline__ long long mul_shift(Split a, Split b, int s)
     const uint32_t r0 = __funnelshift_l(w0, w1, s), r1 = __funnelshift_l(w1, w2, s);
     return (long long)(((uint64_t)r1 << 32) | r0);
 }
+// the same with the lo lo product: every bit of the result's unit
+__device__ __forceinline__ long long mul_shift_all(Split a, Split b, int s)
+{
+    const long long p0 = (long long)a.hi * b.hi;
+    const long long p1 = (long long)a.hi * b.lo + (long long)a.lo * b.hi + (((long long)a.lo * b.lo) >> 32);
+    const long long h = p0 + (p1 >> 32);
+    const uint32_t w0 = (uint32_t)p1, w1 = (uint32_t)h, w2 = (uint32_t)(h >> 32);
+    const uint32_t r0 = __funnelshift_l(w0, w1, s), r1 = __funnelshift_l(w1, w2, s);
+    return (long long)(((uint64_t)r1 << 32) | r0);
+}
 __device__ __forceinline__ long long shl64(long long x, int s)  // 0 <= s < 32
 {
     const uint32_t lo = (uint32_t)x;
@@ -125,22 +144,27 @@ __device__ __forceinline__ long long sar64(long long x, int s)  // 0 <= s < 32
     const int hi = (int)(x >> 32);
     return (long long)(((uint64_t)(uint32_t)(hi >> s) << 32) | __funnelshift_r((uint32_t)x, (uint32_t)hi, s));
 }
-// The group sums d (exact integers) as one integer of unit 2^-60, for W' =
-// 2^e Wint: the weight of group g is 2^(-16 - 8 g + e); p = 20 + e, q = 4 - e.
-template <int NSL>
-__device__ __forceinline__ long long fx_sum(const float (&d)[NSL], int p, int q)
+// (a b) 2^-64 2^(s + d), |d| < 29
+__device__ __forceinline__ long long mul_unit(Split a, Split b, int s, int d)
 {
-    long long a = __float2int_rn(d[3]);
-    a += (long long)__float2int_rn(d[2]) * 256;
-    a += (long long)__float2int_rn(d[1]) * 65536;
-    a += (long long)__float2int_rn(d[0]) * 16777216;
-    long long r = shl64(a, p);
-    if constexpr (NSL > 4) {
-        long long b = (long long)__float2int_rn(d[4]) * 65536;
-        if constexpr (NSL > 5) b += (long long)__float2int_rn(d[5]) * 256;
-        if constexpr (NSL > 6) b += __float2int_rn(d[6]);
-        r += sar64(b, q);
-    }
+    return sar64(mul_shift_all(a, b, s + max(d, 0)), max(-d, 0));
+}
+// The group sums d (exact integers) as one integer of unit 2^(-60 - s), for W' =
+// 2^e Wint: the weight of group g is 2^(-16 - 8 g + e), t = -4 - e - s >= -8.  The
+// sum of the first six groups fits 63 bits (|d_0| < 2^22.5).  left: t may be
+// negative (strong couplings, no shifts; uniform).
+template <int NSL>
+__device__ __forceinline__ long long fx_sum(const float (&d)[NSL], int t, bool left)
+{
+    long long a = __float2int_rn(d[5]);
+    a += (long long)__float2int_rn(d[4]) * 256;
+    a += (long long)__float2int_rn(d[3]) * 65536;
+    a += (long long)__float2int_rn(d[2]) * 16777216;
+    a += (long long)(__float2int_rn(d[0]) * 256 + __float2int_rn(d[1])) << 32;
+    long long r;
+    if (NSL > 6 && left) r = a << -t;  // (e > -4: seven digits)
+    else r = sar64(a, t);
+    if constexpr (NSL > 6) r += __float2int_rn(d[6]) >> min(31, t + 8);
     return r;
 }
 // v 2^ex as a double, rounded to nearest, by its bits; 0 below the normal
@@ -171,6 +195,14 @@ __device__ __forceinline__ long long fixed_of(double x, int sh)
     if (k >= 0) r = m << (k < 12 ? k : 12);
     else if (k > -54) r = (m + (1ull << (-k - 1))) >> -k;
     return b < 0 ? -(long long)r : (long long)r;
+}
+
+// 2^(E + 2), above the modulus of a number whose larger part has the exponent
+// E; 0 below FP32's range.
+__device__ __forceinline__ float above(int E) { return E < -120 ? 0.0f : __int_as_float((min(E, 100) + 129) << 23); }
+__device__ __forceinline__ int exponent_of(double re, double im)  // of the larger part; -1023: zero
+{
+    return (int)((uint32_t)max(__double2hiint(re) & 0x7fffffff, __double2hiint(im) & 0x7fffffff) >> 20) - 1023;
 }
 
 // |x| as a float by its bits, truncated; 0 below and infinity above range.
@@ -236,15 +268,15 @@ __device__ __forceinline__ bool fx_order(FxMma &m, uint32_t &fpar, bool wait, bo
 
 // Digits of four columns (two electrons, re and im) of T into the B operand.
 // With the bias the digits are the bytes of t >> 4; 0x64 above a byte makes
-// the FP16 number 1024 + byte.
+// the FP16 number 1024 + byte.  s0, s1: shifts of the two electrons' entries.
 template <int NSL>
-__device__ __forceinline__ void put_digits(unsigned char *b, int bsl, const long long *t, int nsl = NSL)
+__device__ __forceinline__ void put_digits(unsigned char *b, int bsl, const long long *t, int s0, int s1, int nsl = NSL)
 {
     constexpr long long kBias = (((512ll << 48) + 0x808080808080ll) << 4) + 8;
     uint32_t lo[4], hi[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const long long u = (t[q] + kBias) >> 4;
+        const long long u = (sar64(t[q], q < 2 ? s0 : s1) + kBias) >> 4;
         lo[q] = (uint32_t)u;
         hi[q] = (uint32_t)(u >> 32);
     }
@@ -277,19 +309,23 @@ __device__ __forceinline__ void put_digits(unsigned char *b, int bsl, const long
 
 // One order of the series for this thread's row and columns: the group sums
 // and the Chebyshev sum come from tensor memory, the new digits go to B.
-// sL: shift of the diagonal's product; p, q: shifts of fx_sum; Jk carries
-// the sign of (-i)^(k+1), odd whether it is imaginary.
+// sL: shift of the diagonal's product; t: shift of fx_sum for s = 0; Jk
+// carries the sign of (-i)^(k+1), odd whether it is imaginary; shifts: s of this
+// thread's entries, a byte per electron in shared memory.
 template <int NSL>
 __device__ __forceinline__ void fx_update(long long (&tk)[kFxMaxCols], long long (&tp)[kFxMaxCols], int ncol, int col0,
                                           bool rowok, uint32_t dcol, uint32_t acol, uint32_t NB, unsigned char *brow,
-                                          int bn, int bsl, const Split Ls, int sL, int p, int q, const Split Jk, bool odd)
+                                          int bn, int bsl, const Split Ls, int sL, int t, const Split Jk, bool odd,
+                                          const uchar2 *shifts)
 {
 #pragma unroll
     for (int q4 = 0; q4 < kFxMaxCols; q4 += 4) {
         if (q4 >= ncol) break;
+        const uchar2 s2 = shifts[q4 / 4];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int c = q4 + 2 * h;
+            const int s = h ? s2.y : s2.x;
             float dr[NSL], di[NSL], a0, a1, a2, a3;
 #pragma unroll
             for (int g = 0; g < NSL; ++g) tc::tmem_ld2(dcol + (uint32_t)g * NB + c, dr[g], di[g]);
@@ -299,8 +335,8 @@ __device__ __forceinline__ void fx_update(long long (&tk)[kFxMaxCols], long long
             tp[c] = tk[c];
             tp[c + 1] = tk[c + 1];
             tc::tmem_wait_ld();
-            nr += fx_sum<NSL>(di, p, q);
-            ni -= fx_sum<NSL>(dr, p, q);
+            nr += fx_sum<NSL>(di, t - s, t < 0);
+            ni -= fx_sum<NSL>(dr, t - s, t < 0);
             tk[c] = nr;
             tk[c + 1] = ni;
             const long long jr = mul_shift(split64(nr), Jk, 3), ji = mul_shift(split64(ni), Jk, 3);
@@ -317,7 +353,7 @@ __device__ __forceinline__ void fx_update(long long (&tk)[kFxMaxCols], long long
                          __int_as_float((int)(ai >> 32)));
         }
         const int cb = col0 + q4;
-        if (rowok) put_digits<NSL>(brow + (cb >> 3) * bn + (cb & 7) * 2, bsl, tk + q4);
+        if (rowok) put_digits<NSL>(brow + (cb >> 3) * bn + (cb & 7) * 2, bsl, tk + q4, s2.x, s2.y);
     }
     tc::tmem_wait_st();
 }
@@ -331,6 +367,8 @@ __global__ void __launch_bounds__(kFxThreads, 1)
     __shared__ int s_red[kFxWarps], s_max[8][kFxMaxEl], s_x[kFxMaxEl];
     __shared__ float s_ssq[8][kFxMaxEl];
     __shared__ Split s_J[kChebMax], s_a0[2][kFxMaxEl], s_a1[2][kFxMaxEl];
+    __shared__ int s_as[kFxMaxEl];
+    __shared__ float s_af[kFxMaxEl];
     constexpr int kNan = 0x7fffffff;  // column scale of a column that is not finite
     const int N = s.N, Ne = s.Ne;
     const FxShape f = fx_shape(N);
@@ -396,10 +434,20 @@ __global__ void __launch_bounds__(kFxThreads, 1)
             for (int idx = 2 * e_lo * N + tid; idx < 2 * e_hi * N; idx += kFxThreads) reinterpret_cast<double *>(C)[idx] = nan;
             continue;
         }
-        // W' = 2^e Wint with |Wint| < 2, e in [-19, 4]; nsl digits: the fewest
-        // with 17.5 - 16 - 8 nsl + e <= -56
-        const int e = max(-19, (int)((__double2hiint(wmax) >> 20) & 0x7ff) - 1023);
-        const int nsl = min(kFxS, max(4, (58 + e + 7) / 8));
+        // an entry of T_k changes by at most this much of its column's norm: 2.5
+        // max |W'| sqrt(N) per order (columns normalised below 2, with the
+        // deflated level's share), at most k-fold in T_k; the deflated level's row,
+        // where T_k grows faster, by what k_build_w found
+        const float grow = 1.3f * abs_float(wmax) * sqrtf((float)N) * (float)(K * (K + 1));
+        // couplings so weak that entries that start from zero stay small: every
+        // entry has a unit of its own
+        const bool shifts = grow < 1.0f;  // (max |W'| is below 2^-4 then)
+        uchar2 *s_shift = reinterpret_cast<uchar2 *>(fx_smem + kFxMaxSmem - kFxSlack + 8 * tid);
+        // W' = 2^e Wint with |Wint| < 2, e in [-26, 4]; nsl digits: the fewest
+        // with 17.5 - 16 - 8 nsl + e <= -56 (7 at most); with shifts, 2^-46 of
+        // max |W'|.  Without shifts e is above -18: 6 digits at least
+        const int ew = (int)((__double2hiint(wmax) >> 20) & 0x7ff) - 1023, e = max(-26, ew);
+        const int nsl = shifts ? (e > ew ? 7 : 6) : min(kFxS, (58 + e + 7) / 8);
         // the row's diagonal 2 (L - c) / rho, times 2^(61 - fL) below 2^62
         const int fL = max(1, (int)((__double2hiint(Lc) >> 20) & 0x7ff) - 1023);
         const Split Ls = split64(fixed_of(Lc, 61 - fL));
@@ -462,10 +510,13 @@ __global__ void __launch_bounds__(kFxThreads, 1)
         for (int w = tid; w < nsl * bsl / 16; w += kFxThreads) reinterpret_cast<uint4 *>(B)[w] = make_uint4(0, 0, 0, 0);
         const double *df = s.defl ? s.defl + t * defl_stride(N, Ne) : nullptr;
         const bool defl = df && df[0] != 0.0;
+        const float grow_row = defl && row == N - 1 ? 2.0f * abs_float(df[4]) : grow;
         Split ur = {0, 0}, ui = {0, 0};
+        float uf = 0.0f;  // at least |u_j|
         if (defl && rowok) {
             ur = split64(fixed_of(df[kDeflHead + row], 62));
             ui = split64(fixed_of(df[kDeflHead + N + row], 62));
+            uf = above(exponent_of(df[kDeflHead + row], df[kDeflHead + N + row]));
         }
         Split cc, sc;  // e^{-ic}
         {
@@ -536,7 +587,11 @@ __global__ void __launch_bounds__(kFxThreads, 1)
                 if (defl && tid < ne) {
                     const double *qd = df + kDeflHead + 2 * N + e0 + tid;
                     const double ar = qd[0], ai = qd[Ne], cm = df[2], sm = df[3];
-                    const int sh = 60 - (x == kNan ? 0 : x);
+                    // a in a unit of its own, 2^as finer than the column's
+                    const int ea = exponent_of(ar, ai);
+                    const int as = x == kNan ? 0 : max(0, min(kFxMaxShift, x - ea - 2)), sh = 60 + as - (x == kNan ? 0 : x);
+                    s_as[tid] = as;
+                    s_af[tid] = above(ea - (x == kNan ? 0 : x));
                     s_a0[0][tid] = split64(fixed_of(ar, sh));
                     s_a0[1][tid] = split64(fixed_of(ai, sh));
                     s_a1[0][tid] = split64(fixed_of(fma(cm, ar, sm * ai), sh));  // e^{-i mu} a
@@ -548,19 +603,27 @@ __global__ void __launch_bounds__(kFxThreads, 1)
 #pragma unroll
                 for (int q4 = 0; q4 < kFxMaxCols; q4 += 4) {
                     if (q4 >= ncol) break;
+                    int ups[2] = {0, 0};  // the entries' shifts
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const int el = (col0 + q4) / 2 + h;
                         long long vr = 0, vi = 0;
                         const int x = el < ne ? s_x[el] : kNan;
                         if (rowok && x != kNan) {
-                            vr = fixed_of(__longlong_as_double(tk[q4 + 2 * h]), 60 - x);
-                            vi = fixed_of(__longlong_as_double(tk[q4 + 2 * h + 1]), 60 - x);
+                            const double cr = __longlong_as_double(tk[q4 + 2 * h]), ci = __longlong_as_double(tk[q4 + 2 * h + 1]);
+                            // the entry's shift: |.| 2^(60 + up) stays below 2^61, from
+                            // its size, the deflated level's share and its growth
+                            const float size = above(exponent_of(cr, ci) - x) + (defl ? s_af[el] * uf : 0.0f) + grow_row;
+                            const int up = shifts ? max(0, min(min(kFxMaxShift, -4 - e), 127 - (__float_as_int(size) >> 23))) : 0;
+                            vr = fixed_of(cr, 60 - x + up);
+                            vi = fixed_of(ci, 60 - x + up);
                             if (defl) {  // c - a u
                                 const Split ar = s_a0[0][el], ai = s_a0[1][el];
-                                vr -= mul_shift(ar, ur, 2) - mul_shift(ai, ui, 2);
-                                vi -= mul_shift(ar, ui, 2) + mul_shift(ai, ur, 2);
+                                const int d = up - s_as[el];
+                                vr -= mul_unit(ar, ur, 2, d) - mul_unit(ai, ui, 2, d);
+                                vi -= mul_unit(ar, ui, 2, d) + mul_unit(ai, ur, 2, d);
                             }
+                            ups[h] = up;
                         }
                         tk[q4 + 2 * h] = vr;
                         tk[q4 + 2 * h + 1] = vi;
@@ -570,7 +633,8 @@ __global__ void __launch_bounds__(kFxThreads, 1)
                                      __int_as_float((int)ai), __int_as_float((int)(ai >> 32)));
                     }
                     const int cbq = col0 + q4;
-                    if (rowok) put_digits<kFxS>(brow + (cbq >> 3) * bn + (cbq & 7) * 2, bsl, tk + q4, nsl);
+                    if (rowok) put_digits<kFxS>(brow + (cbq >> 3) * bn + (cbq & 7) * 2, bsl, tk + q4, ups[0], ups[1], nsl);
+                    s_shift[q4 / 4] = make_uchar2((unsigned char)ups[0], (unsigned char)ups[1]);
                 }
                 tc::tmem_wait_st();
             }
@@ -581,12 +645,8 @@ __global__ void __launch_bounds__(kFxThreads, 1)
                 tc::fence_after_sync();
                 if (warp == 0) {
                     if (tc::elect_one()) {
-                        switch (nsl) {
-                        case 4: ok = fx_order<4>(m, fpar, !resident || ord == 0, !resident); break;
-                        case 5: ok = fx_order<5>(m, fpar, !resident || ord == 0, !resident); break;
-                        case 6: ok = fx_order<6>(m, fpar, !resident || ord == 0, !resident); break;
-                        default: ok = fx_order<7>(m, fpar, !resident || ord == 0, !resident); break;
-                        }
+                        ok = nsl == 6 ? fx_order<6>(m, fpar, !resident || ord == 0, !resident)
+                                      : fx_order<7>(m, fpar, !resident || ord == 0, !resident);
                         tc::commit(&done);
                     }
                     __syncwarp();
@@ -619,15 +679,11 @@ __global__ void __launch_bounds__(kFxThreads, 1)
                 tc::fence_after_sync();
                 if (!wact) continue;  // the whole warp holds rows past N
                 // the first order is T_1 = X T_0: half the shifts' values, T_{-1} = 0
-                const int fst = k == 0 ? 1 : 0, sL = 3 + fL - fst, p = 20 + e - fst, q = 4 - e + fst;
+                const int fst = k == 0 ? 1 : 0, sL = 3 + fL - fst, ts = fst - 4 - e;
                 const Split Jk = s_J[k + 1];
                 const bool odd = !(k & 1);
-                switch (nsl) {
-                case 4: fx_update<4>(tk, tp, ncol, col0, rowok, dcol, acol, (uint32_t)NB, brow, bn, bsl, Ls, sL, p, q, Jk, odd); break;
-                case 5: fx_update<5>(tk, tp, ncol, col0, rowok, dcol, acol, (uint32_t)NB, brow, bn, bsl, Ls, sL, p, q, Jk, odd); break;
-                case 6: fx_update<6>(tk, tp, ncol, col0, rowok, dcol, acol, (uint32_t)NB, brow, bn, bsl, Ls, sL, p, q, Jk, odd); break;
-                default: fx_update<7>(tk, tp, ncol, col0, rowok, dcol, acol, (uint32_t)NB, brow, bn, bsl, Ls, sL, p, q, Jk, odd); break;
-                }
+                if (nsl == 6) fx_update<6>(tk, tp, ncol, col0, rowok, dcol, acol, (uint32_t)NB, brow, bn, bsl, Ls, sL, ts, Jk, odd, s_shift);
+                else fx_update<7>(tk, tp, ncol, col0, rowok, dcol, acol, (uint32_t)NB, brow, bn, bsl, Ls, sL, ts, Jk, odd, s_shift);
             }
             if (!ok) {
                 if (tid == 0) atomicOr(&s.status[t], ST_TC_WAIT);
@@ -643,19 +699,20 @@ __global__ void __launch_bounds__(kFxThreads, 1)
                     tc::tmem_wait_ld();
                     const int el = col0 / 2 + q;
                     if (rowok && el < ne) {
-                        const int x = s_x[el];
+                        const int x = s_x[el], up = q & 1 ? s_shift[q / 2].y : s_shift[q / 2].x;
                         const Split ar = split64(((long long)__float_as_int(a1) << 32) | (uint32_t)__float_as_int(a0));
                         const Split ai = split64(((long long)__float_as_int(a3) << 32) | (uint32_t)__float_as_int(a2));
                         long long outr = mul_shift(cc, ar, 2) + mul_shift(sc, ai, 2);
                         long long outi = mul_shift(cc, ai, 2) - mul_shift(sc, ar, 2);
                         if (defl) {
                             const Split br = s_a1[0][el], bi = s_a1[1][el];
-                            outr += mul_shift(br, ur, 3) - mul_shift(bi, ui, 3);
-                            outi += mul_shift(br, ui, 3) + mul_shift(bi, ur, 3);
+                            const int d = up - s_as[el];
+                            outr += mul_unit(br, ur, 3, d) - mul_unit(bi, ui, 3, d);
+                            outi += mul_unit(br, ui, 3, d) + mul_unit(bi, ur, 3, d);
                         }
                         const double nan = __longlong_as_double(0x7ff8000000000000ll);
                         C[(int64_t)(e0 + el) * N + row] = x == kNan ? make_double2(nan, nan)
-                                                                    : make_double2(double_of(outr, x - 61), double_of(outi, x - 61));
+                                                                    : make_double2(double_of(outr, x - 61 - up), double_of(outi, x - 61 - up));
                     }
                 }
             __syncthreads();  // the columns' scales are read before the next block's
@@ -699,12 +756,12 @@ int fx_parts(int Ne, int64_t n, int sms)
 // Where the tensor cores pay: measured against the SIMT kernel k_cheb on the
 // double well (9 orders) and the relaxation model (20 orders), 2048
 // trajectories, Ne = M / 2, ms per step: N = 25 0.84 against 0.66 and 1.65
-// against 1.41; N = 29 0.85 against 0.99 and 1.66 against 2.07; N = 41 1.14
-// against 2.52 and 2.31 against 5.48.  Its cost per trajectory hardly falls
+// against 1.41; N = 29 0.89 against 0.99 and 1.73 against 2.07; N = 41 1.22
+// against 2.52 and 2.45 against 5.48.  Its cost per trajectory hardly falls
 // with Ne below one block of columns, while the SIMT kernel's is N^2 Ne per
 // order: with few electrons the same break-even, N Ne = 28 x 14, holds
-// (N = 101: between 2 and 4 electrons).  The rule takes N and Ne only, so
-// that a batch gives the same bits however it is divided.
+// (N = 101, Ne = 4: 1.17 against 2.84; between 2 and 4).  The rule takes N and
+// Ne only, so that a batch gives the same bits however it is divided.
 bool cheb_fx_eligible(int N, int Ne) { return N >= 28 && N <= 256 && N * Ne >= 28 * 14; }
 
 size_t cheb_fx_work_bytes(int N, int Ne, int64_t max_traj)

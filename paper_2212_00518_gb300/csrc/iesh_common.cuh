@@ -31,10 +31,11 @@ struct ModelDev {
 
 // Device pointers of a context's state (structure of arrays).
 // Deflation record per trajectory, defl_stride doubles: [0] flag, [1] mu,
-// [2] cos mu, [3] sin mu; from kDeflHead the eigenvector u (Re u[N], Im
+// [2] cos mu, [3] sin mu, [4] bound of the top row's part of the deflated
+// columns (unit norms; fixed-point propagator); from kDeflHead the eigenvector u (Re u[N], Im
 // u[N]) and a = u^H c (Re a[Ne], Im a[Ne]), as doubles in FP64 contexts and
 // as packed floats in mixed ones.
-constexpr int kDeflHead = 4;
+constexpr int kDeflHead = 6;
 __host__ __device__ constexpr int64_t defl_stride(int N, int Ne)
 {
     return kDeflHead + 2 * (int64_t)N + 2 * (int64_t)Ne;

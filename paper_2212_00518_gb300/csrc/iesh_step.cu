@@ -256,10 +256,18 @@ __device__ inline bool defl_keep(const DevState &s, int64_t t, bool deflate, dou
         const double *cb = s.cheb + t * kChebStride;
         double tmax = 0.0;
         bool k = deflate && cheb_amplification(cb, mu, tmax) <= amp && rtop <= 8.0 * cb[1] && mu - cb[0] <= 1e6 * cb[1];
-        if (k && s.fx_work) k = tmax * (unit + sqrt(res / den) / (mu - cb[0] - cb[1])) <= kDeflShare;
+        double top = 0.0;
+        if (k && s.fx_work) {
+            const double share = tmax * (unit + sqrt(res / den) / (mu - cb[0] - cb[1]));
+            k = share <= kDeflShare;
+            // the bulk columns' part on the top row, and what grows along u (u_top = 1
+            // before its normalisation)
+            top = sqrt(fmax(den - 1.0, 0.0) / den) + 2.0 * share + 1e-8;
+        }
         if (deflate && !k) cheb_setup(s, t, lo, hi, tol);
         *flag = k;
         if (df) {
+            df[4] = top;
             df[0] = k ? 1.0 : 0.0;
             df[1] = mu;
             if (k) sincos(mu, &df[3], &df[2]);  // once per trajectory
