@@ -320,7 +320,10 @@ const char *iesh_ensemble_last_error(const iesh_ensemble *ens);
  * there and is not applied; its FP32 ratios round differently from the
  * LU's, about 1e-7 relative); IESH_EINVAL otherwise.  The propagator shapes do not change results
  * (each output keeps a fixed summation order).  Used by the autotuner of
- * the Python package. */
+ * the Python package.  iesh_get_kernel_shape gives the shape in use: the
+ * built-in one where none was requested, 0 and 0 for the FP64 tensor-core
+ * propagator, whose blocks follow from the digits that the couplings ask
+ * for. */
 iesh_status iesh_set_kernel_shape(iesh_ctx *ctx, int cheb_ept, int cheb_G, int hop_threads);
 iesh_status iesh_get_kernel_shape(iesh_ctx *ctx, int *cheb_ept, int *cheb_G, int *hop_threads);
 

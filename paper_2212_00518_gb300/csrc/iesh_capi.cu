@@ -741,7 +741,7 @@ iesh_status iesh_get_kernel_shape(iesh_ctx *ctx, int *cheb_ept, int *cheb_G, int
             const int qpt = ctx->N > kCheb32WideMinN ? 2 : 1;
             e = qpt == 2 ? 32 : 4;
             cheb32_shape(ctx->N, ctx->Ne, g, qpt);
-        } else {
+        } else if (!ctx->ds.fx_work) {  // (the FP64 tensor-core kernel: 0, 0)
             cheb_shape(ctx->N, ctx->Ne, e, g);
         }
     }

@@ -4,10 +4,12 @@ Times candidate shapes of the Chebyshev propagator (electrons per thread x
 column groups per CTA) and of the hop kernel (threads per CTA) on a scratch
 context with the same model, precision and batch size, from the caller's
 state, and sets the fastest on the context.  Results do not depend on the
-propagator shape (every output keeps its summation order).  A
-mixed-precision context whose default propagator is the tensor-core kernel
-keeps it (its arithmetic differs from the SIMT shapes); only the hop kernel
-is tuned then.  The hop candidates are the built-in choice (0: in the mixed
+propagator shape (every output keeps its summation order).  A context whose
+default propagator is a tensor-core kernel keeps it and its built-in shape (a
+requested shape only narrows the FP64 kernel's blocks, and the mixed kernels'
+arithmetic differs from the SIMT shapes); only the hop kernel is tuned then.
+For mixed contexts with N > 128 the built-in choice, (0, 0), is among the
+candidates.  The hop candidates are the built-in choice (0: in the mixed
 path the register-resident Gauss-Jordan kernel where it fits) and LU CTAs
 of 256 or 512 threads; the mixed path's two hop algorithms round the FP32
 ratios differently (hop probabilities agree to about 1e-7 relative).
@@ -87,7 +89,12 @@ def autotune(ctx, x, p, occ, C, dt, steps=3, seed=0):
         return prof["propagate"][0], prof["hop"][0]
 
     default = scratch.kernel_shape()[:2]
-    cands = [default] if default[0] in (8, 16) else cheb_candidates(ctx.N, ctx.Ne, precision=ctx.precision)
+    if default[0] in (0, 8, 16):
+        cands = [default]
+    else:
+        cands = cheb_candidates(ctx.N, ctx.Ne, precision=ctx.precision)
+        if ctx.precision == _I.PREC_MIXED:
+            cands = [(0, 0)] + cands
     for ept, G in cands:
         times_cheb[(ept, G)] = trial(ept, G, 0)[0]
     for hop in (0, 256, 512):
