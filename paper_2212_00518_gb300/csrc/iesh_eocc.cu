@@ -28,6 +28,7 @@
 
 #include "../../include/iesh.h"
 #include "iesh_common.cuh"
+#include "iesh_host.h"
 #include "iesh_secular.cuh"
 
 using namespace iesh;
@@ -394,25 +395,15 @@ iesh_status iesh_eocc_forward(iesh_eocc_ctx *c, int64_t B, int precision, const 
     if (e != cudaSuccess) return efail(c, IESH_ECUDA, cudaGetErrorString(e));
     if (precision == IESH_PREC_FP64) {
         const size_t smem = (size_t)5 * threads * sizeof(double) + (size_t)(M + 1) * (2 * sizeof(double) + 2 * sizeof(float2));
-        if (smem > 48 * 1024) {  // a process-wide function attribute: only raised
-            cudaFuncAttributes fa;
-            e = cudaFuncGetAttributes(&fa, k_eocc_fwd<double>);
-            if (e == cudaSuccess && fa.maxDynamicSharedSizeBytes < (int)smem)
-                e = cudaFuncSetAttribute(k_eocc_fwd<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return efail(c, IESH_ECUDA, cudaGetErrorString(e));
-        }
+        if (smem > 48 * 1024) e = allow_max_smem(k_eocc_fwd<double>);
+        if (e != cudaSuccess) return efail(c, IESH_ECUDA, cudaGetErrorString(e));
         k_eocc_fwd<double><<<(unsigned)B, threads, smem, c->stream>>>(
             B, M, Ne, kc, c->eps_d, c->w_d, c->eps_df, c->wsum, (const double *)x, (const double *)theta, (double *)E,
             (double *)saved, status);
     } else if (precision == IESH_PREC_MIXED) {
         const size_t smem = (size_t)5 * threads * sizeof(double) + (size_t)2 * (M + 1) * sizeof(float);
-        if (smem > 48 * 1024) {
-            cudaFuncAttributes fa;
-            e = cudaFuncGetAttributes(&fa, k_eocc_fwd<float>);
-            if (e == cudaSuccess && fa.maxDynamicSharedSizeBytes < (int)smem)
-                e = cudaFuncSetAttribute(k_eocc_fwd<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return efail(c, IESH_ECUDA, cudaGetErrorString(e));
-        }
+        if (smem > 48 * 1024) e = allow_max_smem(k_eocc_fwd<float>);
+        if (e != cudaSuccess) return efail(c, IESH_ECUDA, cudaGetErrorString(e));
         k_eocc_fwd<float><<<(unsigned)B, threads, smem, c->stream>>>(
             B, M, Ne, kc, c->eps_f, c->w_f, c->eps_df, (float)c->wsum, (const float *)x, (const float *)theta, (float *)E,
             (float *)saved, status);

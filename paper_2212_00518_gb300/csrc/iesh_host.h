@@ -10,6 +10,23 @@
 
 namespace iesh {
 
+// Allows a kernel the device's full opt-in shared memory (minus its static
+// shared memory).  The limit is a process-wide function attribute: always the
+// same value, so that host threads that launch different sizes cannot lower
+// each other's between a call and its launch.
+template <class F>
+inline cudaError_t allow_max_smem(F *fn)
+{
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fn);
+    if (e == cudaSuccess && fa.maxDynamicSharedSizeBytes < optin - (int)fa.sharedSizeBytes)
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+    return e;
+}
+
 // Per-class device time of bracketed launches.  With timing on, run()
 // records an event pair around the launch on the given stream; fold()
 // synchronises the last event and accumulates the elapsed times.  Event

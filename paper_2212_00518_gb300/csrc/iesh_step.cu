@@ -15,6 +15,7 @@
 //               momentum rescale (Sec. II B).
 #include "iesh_common.cuh"
 #include "iesh_kernels.h"
+#include "iesh_host.h"
 #include "iesh_secular.cuh"
 #include "iesh_cheb.cuh"
 #include "iesh_hop.cuh"
@@ -1723,22 +1724,9 @@ cudaError_t launch_cheb(const DevState &s, double dt, bool mixed, cudaStream_t s
     return cudaSuccess;
 }
 
-// Allow the hop kernels and the tiled FP32 propagator the device's full opt-in shared memory (minus their
-// static shared memory), so that later launches, including launches under
-// stream capture, need no attribute change.
-template <class F>
-static void allow_max_smem(F *fn)
-{
-    int dev = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, fn) == cudaSuccess && optin > (int)fa.sharedSizeBytes)
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             optin - (int)fa.sharedSizeBytes);
-    cudaGetLastError();
-}
-
+// The hop kernels and the tiled FP32 propagator: set when a context is made, so
+// that later launches, including launches under stream capture, need no
+// attribute change.
 void configure_hop_smem()
 {
     allow_max_smem(k_hop<float2, 512, 1>);
@@ -1751,6 +1739,7 @@ void configure_hop_smem()
     allow_max_smem(k_hop<float2, 256, 4, true>);
     allow_max_smem(k_cheb_f32t<4, 1>);
     allow_max_smem(k_cheb_f32t<4, 2>);
+    cudaGetLastError();
     configure_hop_bj();
     configure_hop_gjl();
 }
@@ -1773,18 +1762,13 @@ cudaError_t launch_hop(const DevState &s, double dt, double mass, uint64_t seed,
     int threads = (2 * smem + 2048 <= 227 * 1024) ? 256 : 512;
     if (s.hop_threads > 0) threads = s.hop_threads;
     // The shared-memory limit is a process-wide function attribute, not a
-    // stream operation.  configure_hop_smem() raises it to the device's opt-in
-    // maximum when a context is created; here it is only ever raised (outside
-    // stream capture), never lowered, so that a small launch cannot take the
-    // room away from a larger one captured later.
+    // stream operation: configure_hop_smem() has raised it when a context was
+    // made; outside stream capture it is raised here too.
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(st, &cs);
     auto go = [&](auto kern) {
         if (cs == cudaStreamCaptureStatusNone) {
-            cudaFuncAttributes fa;
-            if (cudaFuncGetAttributes(&fa, kern) == cudaSuccess &&
-                fa.maxDynamicSharedSizeBytes < (int)smem)
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            allow_max_smem(kern);
             cudaGetLastError();
         }
         kern<<<(unsigned)s.n, threads, smem, st>>>(s, dt, mass, seed, skip_bound, g_out);

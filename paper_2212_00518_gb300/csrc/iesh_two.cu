@@ -1078,17 +1078,6 @@ size_t eigen2_smem(int N, int M, int tpb)
     return (size_t)(2 * M + tpb * per) * sizeof(double) + (size_t)tpb * sizeof(Eig2Slot);
 }
 
-// The shared-memory limit is a process-wide function attribute: only raised.
-template <class F>
-cudaError_t raise_smem(F *fn, size_t bytes)
-{
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, fn);
-    if (e == cudaSuccess && fa.maxDynamicSharedSizeBytes < (int)bytes)
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    return e;
-}
-
 }  // namespace
 
 struct iesh2_ctx {
@@ -1339,8 +1328,8 @@ iesh_status iesh2_create(iesh2_ctx **out, const iesh2_model *model, int precisio
     configure_cheb_fx();
     configure_cheb_tcl();
     // the slots of the eigen kernel can pass the 48 KiB default (N near 65)
-    CU2(raise_smem(k2_eigen<false>, eigen2_smem(N, M, eigen_tpb(N))));
-    CU2(raise_smem(k2_eigen<true>, eigen2_smem(N, M, eigen_tpb(N))));
+    CU2(allow_max_smem(k2_eigen<false>));
+    CU2(allow_max_smem(k2_eigen<true>));
     CU2(cudaMemcpyAsync(eps_d, eps.data(), M * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
     CU2(cudaMemcpyAsync(sq_d, sq.data(), M * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
     // coupling profiles of the dense path: sqrt(w_k), times the Lorentzian
