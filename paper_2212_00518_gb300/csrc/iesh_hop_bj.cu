@@ -496,7 +496,8 @@ bool hop_bj_eligible(int N, int Ne) { return N <= kBjMaxN && Ne >= 1 && Ne <= kB
 
 void configure_hop_bj()
 {
-    // the largest matrix (N = 96, Ne = 48) with its pivot columns, four CTAs per SM
+    // the largest matrix (N = 96, Ne = 48) with its pivot columns: 58 KB, three CTAs
+    // per SM (four up to N = 91, Ne = 45)
     const int most = (int)bj_shape(kBjMaxN, kBjMaxNe, true).total;
     cudaFuncSetAttribute(k_hop_bj<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     cudaFuncSetAttribute(k_hop_bj<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
