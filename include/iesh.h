@@ -73,8 +73,14 @@ typedef enum {
 #define IESH_PROP_AVERAGED 0
 #define IESH_PROP_OVERLAP 1
 
-#define IESH_TRAJ_TC_WAIT 0x20u        /* a tensor-core completion wait gave up (the
-                                          step's coefficients were not updated) */
+#define IESH_TRAJ_TC_WAIT 0x20u        /* a tensor-core completion wait gave up: the
+                                          trajectory's coefficients are not those of
+                                          a step (with N <= 128 in mixed contexts they
+                                          were not updated; the FP64 kernel and the
+                                          mixed one for N > 128 store each block of
+                                          electrons when it is done, so that some
+                                          columns may be a step ahead of the others)
+                                          and its state is to be set again */
 #define IESH_TRAJ_NORM_DRIFT 0x40u     /* after some step, an electron's coefficient
                                           column had | ||c_e||^2 - 1 | above
                                           iesh_options.norm_tol: the propagation
