@@ -170,11 +170,12 @@ __global__ void k_eocc_fwd(int64_t B, int M, int Ne, EoccConst kc, const R *__re
             const Poles<R> pp = {P, pole, wt, nullptr, nullptr, nullptr};
             secular_root<R>(r, pp, hp, Z2, false, R(0), lam, qp, st, &o, &tau);
         }
-        // lam - h_-: the exact offset when the origin pole is h_- itself
-        // lam - h_-: FP64 from the unrounded offset; FP32 from the rounded root,
-        // which is what decides the gradients of the few geometries with a root
-        // within roundings of h_- (up to 4e-5 of a sum over 65536 geometries)
-        const R gap = kF64 ? (o == pos ? tau : (pole[o] - hm) + tau) : lam - hm;
+        // lam - h_-: the exact offset when the origin pole is h_- itself.  FP32
+        // takes it from the rounded root, which is what decides the gradients of
+        // the few geometries with a root within roundings of h_- (up to 4e-5 of a
+        // sum over 65536 geometries), unless that leaves nothing
+        const R offset = o == pos ? tau : (pole[o] - hm) + tau;
+        const R gap = kF64 || lam == hm ? offset : lam - hm;
         const R qm = decoupled ? R(0) : tt * qp / gap;
         const Ads<R> &ad = gs.ad;
         R Q0 = (ad.c[0] * qp - ad.c[1] * qm) * gs.rc;
