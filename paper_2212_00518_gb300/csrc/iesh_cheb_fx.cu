@@ -134,11 +134,6 @@ __device__ __forceinline__ long long mul_shift_all(Split a, Split b, int s)
     const uint32_t r0 = __funnelshift_l(w0, w1, s), r1 = __funnelshift_l(w1, w2, s);
     return (long long)(((uint64_t)r1 << 32) | r0);
 }
-__device__ __forceinline__ long long shl64(long long x, int s)  // 0 <= s < 32
-{
-    const uint32_t lo = (uint32_t)x;
-    return (long long)(((uint64_t)__funnelshift_l(lo, (uint32_t)(x >> 32), s) << 32) | (lo << s));
-}
 __device__ __forceinline__ long long sar64(long long x, int s)  // 0 <= s < 32
 {
     const int hi = (int)(x >> 32);

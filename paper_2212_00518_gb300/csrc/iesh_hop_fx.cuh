@@ -26,7 +26,9 @@
 // that absolute error (10^-6 of them: 10^-10 of the slot's own, where FP64 had
 // 10^-15).  What does not fit -- larger entries or sums, rows that grow further,
 // numbers that are not finite -- goes to the FP64 substitution, from the saved
-// factors; entries and sums are known before the first row.
+// factors; entries and sums are known before the first row.  Of strongly mixed
+// columns (random ones, N = 101) two trajectories in three leave by their sums:
+// 2.98 ms per 2048 trajectories, 1.86 ms where none does.
 //
 // What bounds it: half of the kernel is now the FP64 factorisation; a product
 // is twelve multiply-adds and some twenty other integer instructions.  Four
