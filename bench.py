@@ -41,7 +41,9 @@ TF32_PER_BF16 = 1.1 / 2.25  # nominal dense TF32 : BF16 tensor rate
 # the named batch size, divided by it: the traffic is per-trajectory streams of C and
 # W, so it scales with the batch.  A shape or kernel not in the table reports null.
 DRAM_BYTES_PER_TRAJ = {
-    # no capture of the tensor-core propagators yet
+    # captures of 2048 and 608 trajectories (profiles/iesh_fp64_step_M100.md)
+    ("k_cheb_fx", 101, 50): (343.588864e6 + 200.121600e6) / 2048,
+    ("k_cheb_fx", 201, 100): (1286.355e6 + 593.355776e6) / 608,
 }
 
 
